@@ -133,6 +133,14 @@ pic_status build_entry(const std::vector<pic_sim*>& sims, BatchEntry** out, std:
         g.dim = kv.first.first;
         g.prec = kv.first.second;
         g.push_smem = psm;
+        // one box pitch for the whole group, or 0 (the kernel then reads each member's own)
+        g.push_bx = sims[mem[0]]->h.pb[0];
+        g.push_by = sims[mem[0]]->h.pb[1];
+        for (int i : mem)
+            if (sims[i]->h.pb[0] != g.push_bx || sims[i]->h.pb[1] != g.push_by) {
+                g.push_bx = g.push_by = 0;
+                break;
+            }
         g.yee_smem = ysm;
         g.inc_any = 0;
         g.scan_blocks = n == 1 ? sims[mem[0]]->h.nscanblk : 0;
@@ -150,7 +158,7 @@ pic_status build_entry(const std::vector<pic_sim*>& sims, BatchEntry** out, std:
             g.inc_rows = std::max(g.inc_rows, (c.dim > 1 ? c.n[1] + 1 : 1) * (c.dim > 2 ? c.n[2] + 1 : 1));
         }
         const int nsm = prop.multiProcessorCount;
-        const int bp = std::max(1, sff::prepare_push(g.dim, g.prec, psm));
+        const int bp = std::max(1, sff::prepare_push(g.dim, g.prec, g.push_bx, g.push_by, psm));
         const int byy = std::max(1, sff::prepare_yee(g.dim, g.prec, ysm));
         const int bs = std::max(1, sff::scatter_blocks_per_sm(g.dim, g.prec));
         g.push_grid = (int)std::max<long long>(1, std::min<long long>(nch, (long long)bp * nsm));

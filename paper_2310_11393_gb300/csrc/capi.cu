@@ -833,12 +833,14 @@ pic_status pic_init(const pic_config* cfg_in, const pic_allocator* alloc, void* 
     g.prec = cfg->precision;
     g.push_smem = L.push_smem;
     g.yee_smem = L.yee_smem;
+    g.push_bx = L.pb[0];
+    g.push_by = L.pb[1];
     if (L.push_smem > (size_t)prop.sharedMemPerBlockOptin || L.yee_smem > (size_t)prop.sharedMemPerBlockOptin) {
         fail(s, PIC_EINVAL, "tile needs %zu/%zu bytes of shared memory (max %zu)", L.push_smem, L.yee_smem,
              (size_t)prop.sharedMemPerBlockOptin);
         return cleanup(PIC_EINVAL);
     }
-    const int bp = std::max(1, prepare_push(cfg->dim, cfg->precision, L.push_smem));
+    const int bp = std::max(1, prepare_push(cfg->dim, cfg->precision, L.pb[0], L.pb[1], L.push_smem));
     const int by = std::max(1, prepare_yee(cfg->dim, cfg->precision, L.yee_smem));
     const int bs = std::max(1, scatter_blocks_per_sm(cfg->dim, cfg->precision));
     g.inc_any = h.incgrid;

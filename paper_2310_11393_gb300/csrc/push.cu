@@ -61,18 +61,19 @@ __device__ __forceinline__ int tile_of(const SimDev& S, const int c[3])
     return t;
 }
 
-// order-2 interpolation from a shared-memory box [bz][by][bx]
+// order-2 interpolation from a shared-memory box [bz][by][bx]; f points at the window's first
+// node, bx and bxy are the row and plane pitch (constants in the specialised kernels, so that
+// every load is the base register plus an immediate)
 template <int D, typename R>
-__device__ __forceinline__ R interp(const R* f, int bx, int bxy, const int b0, const int b1, const int b2,
-                                    const R* w0, const R* w1, const R* w2)
+__device__ __forceinline__ R interp(const R* f, const int bx, const int bxy, const R* w0, const R* w1, const R* w2)
 {
     if constexpr (D == 1) {
-        return w0[0] * f[b0] + w0[1] * f[b0 + 1] + w0[2] * f[b0 + 2];
+        return w0[0] * f[0] + w0[1] * f[1] + w0[2] * f[2];
     } else if constexpr (D == 2) {
         R v = R(0);
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            const R* r = f + (b1 + j) * bx + b0;
+            const R* r = f + j * bx;
             v += w1[j] * (w0[0] * r[0] + w0[1] * r[1] + w0[2] * r[2]);
         }
         return v;
@@ -83,7 +84,7 @@ __device__ __forceinline__ R interp(const R* f, int bx, int bxy, const int b0, c
             R vk = R(0);
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
-                const R* r = f + (b2 + k) * bxy + (b1 + j) * bx + b0;
+                const R* r = f + k * bxy + j * bx;
                 vk += w1[j] * (w0[0] * r[0] + w0[1] * r[1] + w0[2] * r[2]);
             }
             v += w2[k] * vk;
@@ -103,13 +104,16 @@ __device__ __forceinline__ R interp(const R* f, int bx, int bxy, const int b0, c
 // FP32 add is a compare-and-swap loop with a round trip per attempt); zero contributions are
 // added too (no test).  The box is turned back into FP32 before its TMA reduce-add; each
 // contribution's rounding is at most 2^-30 max(N, 256) w_max.  FP64 keeps double sums.
-__device__ __forceinline__ void jdep(float* a, float v, float q)
+// Each contribution is a product of a factor c along the current's own axis, scaled by q, and a
+// transverse weight w: the product, its scaling and its rounding are the one FMA.
+__device__ __forceinline__ void jdep(float* a, float c, float w)
 {
-    const float f = fmaf(v, q, 12582912.0f);
+    const float f = fmaf(c, w, 12582912.0f);
     atomicAdd(reinterpret_cast<int*>(a), __float_as_int(f) - 0x4B400000);
 }
-__device__ __forceinline__ void jdep(double* a, double v, double)
+__device__ __forceinline__ void jdep(double* a, double c, double w)
 {
+    const double v = c * w;
     if (v != 0.0) atomicAdd(a, v);
 }
 constexpr float JQ_RANGE = 536870912.0f;   // 2^29
@@ -224,41 +228,6 @@ __device__ __forceinline__ void higuera_cary_update(R u[3], const R E[3], const 
     for (int d = 0; d < 3; ++d) u[d] = R(2) * ub[d] - um[d] + h * E[d];
 }
 
-// Frame count of a particle that lands in cell cn of the tile at offset rel (-1, 0, 1 per
-// axis) from the work item's tile T0: every neighbour of that tile whose one-cell frame
-// holds cn (cn on the tile's first cell along an axis: the neighbour below; on its last:
-// the neighbour above; and their combinations along several axes) gets one count, in a
-// shared-memory histogram over tile offsets -2..2 per axis from the work item's tile.
-// Tiles are at least two cells wide, so a cell is first or last along an axis, not both.
-template <int D>
-__device__ __forceinline__ void frame_count(const SimDev& S, const int cn[3], const int T0[3], const int rel[3],
-                                            int* s_frame)
-{
-    int f[3] = {0, 0, 0}, base = 0;
-    bool any = false;
-    constexpr int W[3] = {1, 5, 25};
-#pragma unroll
-    for (int d = 0; d < D; ++d) {
-        const int l = cn[d] - (T0[d] + rel[d] * S.pt[d]);
-        f[d] = l == 0 ? -1 : (l == S.pt[d] - 1 ? 1 : 0);
-        any = any || f[d] != 0;
-        base += (rel[d] + 2) * W[d];
-    }
-    if (!any) return;
-#pragma unroll
-    for (int m = 1; m < (1 << D); ++m) {
-        int idx = base;
-        bool ok = true;
-#pragma unroll
-        for (int d = 0; d < D; ++d)
-            if ((m >> d) & 1) {
-                ok = ok && f[d] != 0;
-                idx += f[d] * W[d];
-            }
-        if (ok) atomicAdd(&s_frame[idx], 1);
-    }
-}
-
 // Threads of a push block and blocks per SM the registers are budgeted for.  The 3D FP32
 // push shares its 101 KB box (16x8x4 tiles) among 512 threads at 64 registers: two blocks
 // keep 32 warps per SM busy instead of 16 with 256-thread blocks at 128 registers.
@@ -294,7 +263,20 @@ __device__ __forceinline__ ChunkRef chunk_of_one(const SimDev& S, const int* __r
 // `sorting`: this step's re-sort orders the tiles by cell; then the simulations that have a
 // cell sort are pushed in place (k_scatter places them) and the others straight into the
 // other buffer set like every step.
-template <int D, typename R, bool ONE>
+// BX, BY: row pitch and rows per plane of the box when they are compile-time constants (the
+// specialised kernels, see with_pitch), 0 when they come from the descriptor.
+//
+// What bounds the FP32 push: the shared-memory pipe (3D at the focus: 63 % of its wavefronts in
+// use, 3.0 per gather load and 3.6 per current add of a warp, issue slots 49 %).  Lanes of a warp
+// share banks and, in a bunched plasma, cells, so an add that only some lanes need costs fewer
+// wavefronts when the others leave it out: with the nodes of the deposit taken as three core nodes
+// per axis plus one for the lanes that cross (instead of a window of four for a warp with any
+// crossing lane) the adds' wavefronts fell from 36.2 M to 22.7 M in the 3D push of 2.1 M electrons.
+// Fewer instructions beside it (the transverse weight as A A' + DS DS'/12, one FMA per
+// contribution, loads and adds at immediate offsets, one count per particle from which the tile
+// and frame counts follow): 3D push of 16.8 M electrons (tiles 16x8x4) 2.01 -> 1.84 ms, of 2.0 M
+// (tiles 8x8x8) 0.534 -> 0.450 ms, 2D of 2.1 M (tiles 32x16) 0.137 -> 0.133 ms.
+template <int D, typename R, bool ONE, int BX, int BY>
 __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const SimDev& one, int nsims,
                                           const int* __restrict__ gprefix, int* __restrict__ counter, int sorting)
 {
@@ -304,6 +286,7 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
     __shared__ int s_hist[27];
     constexpr int NFR = D == 1 ? 5 : (D == 2 ? 25 : 125);
     __shared__ int s_frame[NFR];
+    __shared__ int s_cls[NFR];       // particles by the place of their new cell along each axis
     __shared__ PhaseRef<R> s_pref;
     const int tid = threadIdx.x, nth = blockDim.x;
     if (tid == 0) {
@@ -338,7 +321,7 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
             if constexpr (D > 2) tc[2] = t;
         }
         const int T0[3] = {tc[0] * S.pt[0], tc[1] * S.pt[1], tc[2] * S.pt[2]};
-        const int bx = S.pb[0], by = D > 1 ? S.pb[1] : 1, bz = D > 2 ? S.pb[2] : 1;
+        const int bx = BX > 0 ? BX : S.pb[0], by = D > 1 ? (BY > 0 ? BY : S.pb[1]) : 1, bz = D > 2 ? S.pb[2] : 1;
         const int bxy = bx * by, bvol = bxy * bz;
         R* Fs = reinterpret_cast<R*>(smem_raw);   // [6][bz][by][bx]: Ex Ey Ez Bx By Bz at step n
         R* Js = reinterpret_cast<R*>(smem_raw + round128(6 * bvol * sizeof(R)));   // [3][bz][by][bx]
@@ -359,7 +342,7 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
         }
         for (int i = tid; i < 3 * bvol; i += nth) Js[i] = R(0);
         if (tid < 27) s_hist[tid] = 0;
-        for (int i = tid; i < NFR; i += nth) s_frame[i] = 0;
+        for (int i = tid; i < NFR; i += nth) s_frame[i] = s_cls[i] = 0;
         const bool ok = mbar_wait_bounded(&bar, phase);
         phase ^= 1u;
         if (__syncthreads_or(!ok)) {
@@ -439,12 +422,19 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
                 for (int d = 0; d < 3; ++d) u[d] = reinterpret_cast<const R*>(S.mom[par][d])[p];
                 wt = reinterpret_cast<const R*>(S.wgt[par])[p];
                 R E[3], B[3];
-                E[0] = Ei[0] + interp<D, R>(Fs + 0 * bvol, bx, bxy, ld[0], lp[1], lp[2], Wd[0], Wp[1], Wp[2]);
-                E[1] = Ei[1] + interp<D, R>(Fs + 1 * bvol, bx, bxy, lp[0], ld[1], lp[2], Wp[0], Wd[1], Wp[2]);
-                E[2] = Ei[2] + interp<D, R>(Fs + 2 * bvol, bx, bxy, lp[0], lp[1], ld[2], Wp[0], Wp[1], Wd[2]);
-                B[0] = Bi[0] + interp<D, R>(Fs + 3 * bvol, bx, bxy, lp[0], ld[1], ld[2], Wp[0], Wd[1], Wd[2]);
-                B[1] = Bi[1] + interp<D, R>(Fs + 4 * bvol, bx, bxy, ld[0], lp[1], ld[2], Wd[0], Wp[1], Wd[2]);
-                B[2] = Bi[2] + interp<D, R>(Fs + 5 * bvol, bx, bxy, ld[0], ld[1], lp[2], Wd[0], Wd[1], Wp[2]);
+                // first node of the window of a component: dual (half-cell) axes given by bits of dual
+                auto win = [&](int comp, int dual) {
+                    int i = comp * bvol + ((dual & 1) ? ld[0] : lp[0]);
+                    if constexpr (D > 1) i += ((dual & 2) ? ld[1] : lp[1]) * bx;
+                    if constexpr (D > 2) i += ((dual & 4) ? ld[2] : lp[2]) * bxy;
+                    return Fs + i;
+                };
+                E[0] = Ei[0] + interp<D, R>(win(0, 1), bx, bxy, Wd[0], Wp[1], Wp[2]);
+                E[1] = Ei[1] + interp<D, R>(win(1, 2), bx, bxy, Wp[0], Wd[1], Wp[2]);
+                E[2] = Ei[2] + interp<D, R>(win(2, 4), bx, bxy, Wp[0], Wp[1], Wd[2]);
+                B[0] = Bi[0] + interp<D, R>(win(3, 6), bx, bxy, Wp[0], Wd[1], Wd[2]);
+                B[1] = Bi[1] + interp<D, R>(win(4, 5), bx, bxy, Wd[0], Wp[1], Wd[2]);
+                B[2] = Bi[2] + interp<D, R>(win(5, 3), bx, bxy, Wd[0], Wd[1], Wp[2]);
 
                 // ---- momentum update, charge -1, mass 1 (u^{n-1/2} -> u^{n+1/2}) ----
                 if (S.pusher == 1) vay_update<R>(u, E, B, hq);
@@ -454,19 +444,18 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
                 const R v[3] = {u[0] * ig, u[1] * ig, u[2] * ig};
 
                 // ---- Esirkepov deposition of the move ----
-                // Per axis the old shape covers the old nearest node and its two neighbours; the
-                // new shape is shifted by sh in {-1, 0, 1} nodes (|move| < 1 cell), so both fit a
-                // window of four nodes starting one below the old support when sh = -1 and at it
-                // otherwise.  S0 / DS: old shape / shape change on that window.  Along the
-                // current's own axis the window's last partial sum is the total charge change,
-                // zero: one node fewer carries that component.  When no lane of the warp changes
-                // its nearest node along an axis (sh = 0 everywhere: most steps of most
-                // electrons), the window's fourth node is zero for every lane and the loops stop
-                // at three nodes on that axis (a warp-uniform bound).
-                R S0[3][4], DS[3][4];
-                int jw[3] = {0, 0, 0};
+                // Per axis the old shape covers the old nearest node and its two neighbours (the
+                // core nodes m = 0, 1, 2); the new shape is shifted by sh in {-1, 0, 1} nodes
+                // (|move| < 1 cell), so a lane that changes its nearest node has one node more, two
+                // past the middle one on the side it moves to (m = 3).  A / DS: mean of old and new
+                // shape / shape change on these nodes.  Along the current's own axis the running sum
+                // of DS ends at zero, so that component has the core nodes 0 and 1, and a lane that
+                // crosses a third, with the charge -/+ DS[3] that it carries over it.  The additions
+                // at nodes that only crossing lanes have are left to those lanes.
+                R A[3][4], DS[3][4];
+                int jb = 0;                                  // core node (0, 0, 0) in the box
+                bool cross[3] = {false, false, false}, low[3] = {false, false, false};
                 R mv[3] = {R(0), R(0), R(0)};
-                bool cross[3] = {false, false, false};
 #pragma unroll
                 for (int d = 0; d < D; ++d) {
                     mv[d] = dtdx * v[d];
@@ -480,14 +469,17 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
                     shape2(d1, w1);
                     const bool lo = sh < 0, hi = sh > 0;
                     cross[d] = sh != 0;
-                    const R o0[4] = {lo ? R(0) : w0[0], lo ? w0[0] : w0[1], lo ? w0[1] : w0[2], lo ? w0[2] : R(0)};
-                    const R n1[4] = {hi ? R(0) : w1[0], hi ? w1[0] : w1[1], hi ? w1[1] : w1[2], hi ? w1[2] : R(0)};
+                    low[d] = lo;
+                    const R n1[4] = {hi ? R(0) : (lo ? w1[1] : w1[0]), hi ? w1[0] : (lo ? w1[2] : w1[1]),
+                                     hi ? w1[1] : (lo ? R(0) : w1[2]), hi ? w1[2] : (lo ? w1[0] : R(0))};
 #pragma unroll
-                    for (int m = 0; m < 4; ++m) {
-                        S0[d][m] = o0[m];
-                        DS[d][m] = n1[m] - o0[m];
+                    for (int m = 0; m < 3; ++m) {
+                        DS[d][m] = n1[m] - w0[m];
+                        A[d][m] = w0[m] + R(0.5) * DS[d][m];
                     }
-                    jw[d] = c[d] + h0 - (lo ? 2 : 1) - T0[d] + hx[d];
+                    DS[d][3] = n1[3];
+                    A[d][3] = R(0.5) * n1[3];
+                    jb += (c[d] + h0 - 1 - T0[d] + hx[d]) * (d == 0 ? 1 : (d == 1 ? bx : bxy));
                 }
                 // ---- move: carry the offset into the cell index; removal near the faces.
                 // Done before the deposit's loops below, so that across them only the new cell,
@@ -522,19 +514,20 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
                         atomicOr(&st->status, (unsigned)FLAG_EXIT_OVERFLOW);
                     }
                 } else {
-                    // destination tile relative to this one (a move is under one cell per axis)
-                    int hidx = 0, mul = 1, tg = 0, tmul = 1;
-                    int rel[3] = {0, 0, 0};
+                    // destination tile relative to this one (a move is under one cell per axis),
+                    // and the cell's place along each axis: 0 in the tile below, 1 first cell,
+                    // 2 inside, 3 last cell, 4 in the tile above
+                    int cls = 0, cmul = 1, tg = 0, tmul = 1;
 #pragma unroll
                     for (int d = 0; d < D; ++d) {
-                        rel[d] = cn[d] < T0[d] ? -1 : (cn[d] >= T0[d] + S.pt[d] ? 1 : 0);
-                        hidx += (rel[d] + 1) * mul;
-                        mul *= 3;
-                        tg += (tc[d] + rel[d]) * tmul;
+                        const int l = cn[d] - T0[d];
+                        const int k = l < 0 ? 0 : (l >= S.pt[d] ? 4 : (l == 0 ? 1 : (l == S.pt[d] - 1 ? 3 : 2)));
+                        cls += k * cmul;
+                        cmul *= 5;
+                        tg += (tc[d] + (k == 0 ? -1 : (k == 4 ? 1 : 0))) * tmul;
                         tmul *= S.npt[d];
                     }
-                    atomicAdd(&s_hist[hidx], 1);
-                    frame_count<D>(S, cn, T0, rel, s_frame);
+                    atomicAdd(&s_cls[cls], 1);
                     ncl = encode_cell<D>(S, cn);
                     tdst = tg;
                 }
@@ -545,124 +538,82 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
 #pragma unroll
                     for (int d = 0; d < 3; ++d) reinterpret_cast<R*>(S.mom[par][d])[p] = u[d];
                 }
-                // ---- the deposit on the windows set up above ----
-                // window width per axis over the lanes running here (each lane's own vote is in
-                // its mask, so its width covers its own window whatever the warp's convergence)
-                const unsigned am = __activemask();
-                int nw[3] = {4, 4, 4};
+                // ---- the deposit on the nodes set up above ----
+                // Esirkepov's transverse weight S0 S0' + (DS S0' + S0 DS')/2 + DS DS'/3 is
+                // A A' + DS DS'/12; along the current's own axis the factor is the running sum
+                // of DS, times the scale of the fixed point (FP32)
+                const R qs = sizeof(R) == 4 ? jq : R(1);
+                const R cw = jfac * wt * qs;
+                const R t12 = R(1) / R(12);
+                const int pitch[3] = {1, bx, bxy};
+                int ex[3];                       // offset of the extra node from core node 0
 #pragma unroll
-                for (int d = 0; d < D; ++d) nw[d] = __any_sync(am, cross[d]) ? 4 : 3;
-                R* Jx = Js;
-                R* Jy = Js + bvol;
-                R* Jz = Js + 2 * bvol;
-                const R cw = jfac * wt;
-                const R third = R(1) / R(3);
+                for (int d = 0; d < 3; ++d) ex[d] = low[d] ? -pitch[d] : 3 * pitch[d];
+                // node m of axis d as an offset from core node 0
+                auto at = [&](int d, int m) { return m < 3 ? m * pitch[d] : ex[d]; };
+                // the current along axis d at the nodes of transverse weight w from f on
+                auto line = [&](int d, R* f, const R C[3], R w) {
+                    jdep(f, C[0], w);
+                    jdep(f + pitch[d], C[1], w);
+                    if (cross[d]) jdep(f + (low[d] ? -pitch[d] : 2 * pitch[d]), C[2], w);
+                };
+                auto run_sum = [&](int d, R C[3]) {
+                    C[0] = cw * (DS[d][0] + (low[d] ? DS[d][3] : R(0)));
+                    C[1] = C[0] + cw * DS[d][1];
+                    C[2] = cw * (low[d] ? DS[d][3] : -DS[d][3]);
+                };
                 if constexpr (D == 1) {
-                    R acc = R(0);
+                    R C[3];
+                    run_sum(0, C);
+                    R* f = Js + jb;
+                    line(0, f, C, R(1));
+                    const R qy = -wt * v[1] * qs, qz = -wt * v[2] * qs;
 #pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        if (a >= nw[0] - 1) break;
-                        acc += cw * DS[0][a];
-                        jdep(&Jx[jw[0] + a], acc, jq);
-                    }
-#pragma unroll
-                    for (int a = 0; a < 4; ++a) {
-                        if (a >= nw[0]) break;
-                        const R f = S0[0][a] + R(0.5) * DS[0][a];
-                        jdep(&Jy[jw[0] + a], -wt * v[1] * f, jq);
-                        jdep(&Jz[jw[0] + a], -wt * v[2] * f, jq);
-                    }
+                    for (int m = 0; m < 4; ++m)
+                        if (m < 3 || cross[0]) {
+                            jdep(f + bvol + at(0, m), qy, A[0][m]);
+                            jdep(f + 2 * bvol + at(0, m), qz, A[0][m]);
+                        }
                 } else if constexpr (D == 2) {
 #pragma unroll
-                    for (int b = 0; b < 4; ++b) {
-                        if (b >= nw[1]) break;
-                        const R fy = S0[1][b] + R(0.5) * DS[1][b];
-                        R acc = R(0);
+                    for (int d = 0; d < 2; ++d) {
+                        const int t = 1 - d;
+                        R C[3];
+                        run_sum(d, C);
+                        R* f = Js + d * bvol + jb;
 #pragma unroll
-                        for (int a = 0; a < 3; ++a) {
-                            if (a >= nw[0] - 1) break;
-                            acc += cw * DS[0][a] * fy;
-                            jdep(&Jx[(jw[1] + b) * bx + jw[0] + a], acc, jq);
-                        }
+                        for (int m = 0; m < 4; ++m)
+                            if (m < 3 || cross[t]) line(d, f + at(t, m), C, A[t][m]);
                     }
-#pragma unroll
-                    for (int a = 0; a < 4; ++a) {
-                        if (a >= nw[0]) break;
-                        const R fx = S0[0][a] + R(0.5) * DS[0][a];
-                        R acc = R(0);
-#pragma unroll
-                        for (int b = 0; b < 3; ++b) {
-                            if (b >= nw[1] - 1) break;
-                            acc += cw * DS[1][b] * fx;
-                            jdep(&Jy[(jw[1] + b) * bx + jw[0] + a], acc, jq);
-                        }
-                    }
-                    const R qv = -wt * v[2];
+                    const R qz = -wt * v[2] * qs;
+                    R* f = Js + 2 * bvol + jb;
 #pragma unroll
                     for (int b = 0; b < 4; ++b) {
-                        if (b >= nw[1]) break;
+                        if (b == 3 && !cross[1]) break;
+                        const R db = t12 * DS[1][b];
 #pragma unroll
-                        for (int a = 0; a < 4; ++a) {
-                            if (a >= nw[0]) break;
-                            const R wz = S0[0][a] * S0[1][b] + R(0.5) * DS[0][a] * S0[1][b] +
-                                         R(0.5) * S0[0][a] * DS[1][b] + third * DS[0][a] * DS[1][b];
-                            jdep(&Jz[(jw[1] + b) * bx + jw[0] + a], qv * wz, jq);
-                        }
+                        for (int a = 0; a < 4; ++a)
+                            if (a < 3 || cross[0])
+                                jdep(f + at(1, b) + at(0, a), qz, A[0][a] * A[1][b] + DS[0][a] * db);
                     }
                 } else {
 #pragma unroll
-                    for (int cc = 0; cc < 4; ++cc) {
-                        if (cc >= nw[2]) break;
+                    for (int d = 0; d < 3; ++d) {
+                        const int t = d == 0 ? 1 : 0, z = d == 2 ? 1 : 2;       // transverse axes
+                        R C[3];
+                        run_sum(d, C);
+                        R* f = Js + d * bvol + jb;
 #pragma unroll
-                        for (int b = 0; b < 4; ++b) {
-                            if (b >= nw[1]) break;
-                            const R fyz = S0[1][b] * S0[2][cc] + R(0.5) * DS[1][b] * S0[2][cc] +
-                                          R(0.5) * S0[1][b] * DS[2][cc] + third * DS[1][b] * DS[2][cc];
-                            R acc = R(0);
+                        for (int k = 0; k < 4; ++k) {
+                            if (k == 3 && !cross[z]) break;
+                            const R dk = t12 * DS[z][k];
 #pragma unroll
-                            for (int a = 0; a < 3; ++a) {
-                                if (a >= nw[0] - 1) break;
-                                acc += cw * DS[0][a] * fyz;
-                                jdep(&Jx[(jw[2] + cc) * bxy + (jw[1] + b) * bx + jw[0] + a], acc, jq);
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int cc = 0; cc < 4; ++cc) {
-                        if (cc >= nw[2]) break;
-#pragma unroll
-                        for (int a = 0; a < 4; ++a) {
-                            if (a >= nw[0]) break;
-                            const R fxz = S0[0][a] * S0[2][cc] + R(0.5) * DS[0][a] * S0[2][cc] +
-                                          R(0.5) * S0[0][a] * DS[2][cc] + third * DS[0][a] * DS[2][cc];
-                            R acc = R(0);
-#pragma unroll
-                            for (int b = 0; b < 3; ++b) {
-                                if (b >= nw[1] - 1) break;
-                                acc += cw * DS[1][b] * fxz;
-                                jdep(&Jy[(jw[2] + cc) * bxy + (jw[1] + b) * bx + jw[0] + a], acc, jq);
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int b = 0; b < 4; ++b) {
-                        if (b >= nw[1]) break;
-#pragma unroll
-                        for (int a = 0; a < 4; ++a) {
-                            if (a >= nw[0]) break;
-                            const R fxy = S0[0][a] * S0[1][b] + R(0.5) * DS[0][a] * S0[1][b] +
-                                          R(0.5) * S0[0][a] * DS[1][b] + third * DS[0][a] * DS[1][b];
-                            R acc = R(0);
-#pragma unroll
-                            for (int cc = 0; cc < 3; ++cc) {
-                                if (cc >= nw[2] - 1) break;
-                                acc += cw * DS[2][cc] * fxy;
-                                jdep(&Jz[(jw[2] + cc) * bxy + (jw[1] + b) * bx + jw[0] + a], acc, jq);
-                            }
+                            for (int b = 0; b < 4; ++b)
+                                if (b < 3 || cross[t])
+                                    line(d, f + at(z, k) + at(t, b), C, A[t][b] * A[z][k] + DS[t][b] * dk);
                         }
                     }
                 }
-
             }
             // ---- placement into the destination tile's slots of the other buffer set (all
             // lanes of the warp take part in the reservation) ----
@@ -688,6 +639,38 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
         __syncthreads();
 
         // ---- current flush and destination-tile counts ----
+        // Tile counts and frame counts from the counts by place: a cell of place k sits in the
+        // tile at offset -1, 0 or 1 per axis, and in the one-cell frames of the neighbours of that
+        // tile across the faces it lies on (the cell reached from below is its tile's last one,
+        // the cell reached above its tile's first one; tiles are at least two cells wide), by any
+        // non-empty set of these faces' axes.  s_frame: tile offsets -2 .. 2 per axis.
+        if (tid < NFR && s_cls[tid] > 0) {
+            constexpr int W5[3] = {1, 5, 25}, W3[3] = {1, 3, 9};
+            const int v = s_cls[tid];
+            int k = tid, hidx = 0, base = 0, f[3] = {0, 0, 0};
+#pragma unroll
+            for (int d = 0; d < D; ++d) {
+                const int pl = k % 5;
+                k /= 5;
+                const int rel = pl == 0 ? -1 : (pl == 4 ? 1 : 0);
+                f[d] = pl == 2 ? 0 : ((pl & 1) ? pl - 2 : -rel);
+                hidx += (rel + 1) * W3[d];
+                base += (rel + 2) * W5[d];
+            }
+            atomicAdd(&s_hist[hidx], v);
+#pragma unroll
+            for (int m = 1; m < (1 << D); ++m) {
+                int idx = base;
+                bool ok = true;
+#pragma unroll
+                for (int d = 0; d < D; ++d)
+                    if ((m >> d) & 1) {
+                        ok = ok && f[d] != 0;
+                        idx += f[d] * W5[d];
+                    }
+                if (ok) atomicAdd(&s_frame[idx], v);
+            }
+        }
         if constexpr (sizeof(R) == 4) {
             // fixed point back to FP32, in place
             const float inv = (float)max(p1 - p0, 256) * wmax * (1.0f / JQ_RANGE);
@@ -714,6 +697,7 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
                 }
             }
         }
+        if constexpr (sizeof(R) == 8) __syncthreads();      // (FP32: the barriers of the flush)
         constexpr int NH = D == 1 ? 3 : (D == 2 ? 9 : 27);
         if (tid < NH && s_hist[tid] > 0) {
             int h = tid, nt = 0, mul = 1;
@@ -749,20 +733,20 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
     if (tid == 0) bulk_wait0();
 }
 
-template <int D, typename R>
+template <int D, typename R, int BX, int BY>
 __global__ void __launch_bounds__(push_threads<D, R>(), push_min_blocks<D, R>())
     k_push(const SimDev* __restrict__ sims, int nsims, const int* __restrict__ gprefix, int* __restrict__ counter,
            int sorting)
 {
-    push_body<D, R, false>(sims, *sims, nsims, gprefix, counter, sorting);
+    push_body<D, R, false, BX, BY>(sims, *sims, nsims, gprefix, counter, sorting);
 }
 
 // one simulation: the descriptor by value in the kernel's parameters
-template <int D, typename R>
+template <int D, typename R, int BX, int BY>
 __global__ void __launch_bounds__(push_threads<D, R>(), push_min_blocks<D, R>())
     k_push1(const __grid_constant__ SimDev one, const int* __restrict__ gprefix, int* __restrict__ counter, int sorting)
 {
-    push_body<D, R, true>(nullptr, one, 1, gprefix, counter, sorting);
+    push_body<D, R, true, BX, BY>(nullptr, one, 1, gprefix, counter, sorting);
 }
 
 // Block-wide exclusive scan of one int per thread (blockDim a multiple of 32, <= 1024).
@@ -1416,15 +1400,44 @@ __global__ void k_place_slab(const SimDev* __restrict__ sim, long long n, int pp
 }
 
 // ---- host launch wrappers ------------------------------------------------------------
+// f.template operator()<BX, BY>() with the constant box pitch of the group, or <0, 0>: the box
+// shapes of the default tiles and of the tiles that the autotuner mostly picks (2D: tiles 16, 32
+// and 64 cells wide; 3D: 8 or 16 cells wide and 8 cells high).  Box extents: tile + 8 along x,
+// tile + 5 along y.
+template <int D, typename R, typename F>
+static void with_pitch(int bx, int by, F f)
+{
+    if constexpr (D == 2 && sizeof(R) == 4) {
+        if (bx == 24) return f.template operator()<24, 0>();
+        if (bx == 40) return f.template operator()<40, 0>();
+        if (bx == 72) return f.template operator()<72, 0>();
+    } else if constexpr (D == 3 && sizeof(R) == 4) {
+        if (bx == 16 && by == 13) return f.template operator()<16, 13>();
+        if (bx == 24 && by == 13) return f.template operator()<24, 13>();
+    }
+    f.template operator()<0, 0>();
+}
+
+template <int D, typename R>
+struct PushLaunch {
+    const Group& g;
+    bool sorting;
+    cudaStream_t s;
+    template <int BX, int BY>
+    void operator()() const
+    {
+        if (g.one)
+            k_push1<D, R, BX, BY><<<g.push_grid, push_threads<D, R>(), g.push_smem, s>>>(
+                *g.one, g.gprefix, g.counters + 0, sorting ? 1 : 0);
+        else
+            k_push<D, R, BX, BY><<<g.push_grid, push_threads<D, R>(), g.push_smem, s>>>(
+                g.sims, g.nsims, g.gprefix, g.counters + 0, sorting ? 1 : 0);
+    }
+};
 template <int D, typename R>
 static void push_t(const Group& g, bool sorting, cudaStream_t s)
 {
-    if (g.one)
-        k_push1<D, R><<<g.push_grid, push_threads<D, R>(), g.push_smem, s>>>(*g.one, g.gprefix, g.counters + 0,
-                                                                              sorting ? 1 : 0);
-    else
-        k_push<D, R><<<g.push_grid, push_threads<D, R>(), g.push_smem, s>>>(g.sims, g.nsims, g.gprefix,
-                                                                             g.counters + 0, sorting ? 1 : 0);
+    with_pitch<D, R>(g.push_bx, g.push_by, PushLaunch<D, R>{g, sorting, s});
 }
 template <int D, typename R>
 static void cellsort_t(const Group& g, cudaStream_t s)
@@ -1543,19 +1556,31 @@ void launch_sort_linear(const SimDev* sim, int dim, int prec, long long n, cudaS
 }
 
 template <int D, typename R>
-static void attr_push(size_t smem, int* out)
+struct PushAttr {
+    size_t smem;
+    int* out;
+    template <int BX, int BY>
+    void operator()() const
+    {
+        auto k = k_push<D, R, BX, BY>;
+        auto k1 = k_push1<D, R, BX, BY>;
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        int a = 0, b = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k, push_threads<D, R>(), smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k1, push_threads<D, R>(), smem);
+        *out = std::min(a, b);
+    }
+};
+template <int D, typename R>
+static void attr_push(int bx, int by, size_t smem, int* out)
 {
-    cudaFuncSetAttribute(k_push<D, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(k_push1<D, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    int a = 0, b = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_push<D, R>, push_threads<D, R>(), smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_push1<D, R>, push_threads<D, R>(), smem);
-    *out = std::min(a, b);
+    with_pitch<D, R>(bx, by, PushAttr<D, R>{smem, out});
 }
-int prepare_push(int dim, int prec, size_t smem)
+int prepare_push(int dim, int prec, int bx, int by, size_t smem)
 {
     int b = 0;
-    SFF_DISPATCH(dim, prec, attr_push, smem, &b);
+    SFF_DISPATCH(dim, prec, attr_push, bx, by, smem, &b);
     return b;
 }
 

@@ -31,6 +31,7 @@ struct Group {
     int* counters;         // device: [0] push, [1] scatter, [2] field solver
     int dim, prec;
     size_t push_smem, yee_smem;
+    int push_bx, push_by;  // row pitch and rows per plane of the push box (0: they differ between members)
     int push_grid, yee_grid, scatter_grid;
     int inc_any, inc_segs, inc_rows;   // incident field on the grid: any member, x segments, rows
     int scan_blocks;                   // single simulation: blocks of the multi-block tile scan
@@ -113,7 +114,7 @@ inline bool yee_tile_active(const SimDev& h, int dim, int t)
 }
 
 // kernel attributes (dynamic shared memory opt-in); returns blocks per SM
-int prepare_push(int dim, int prec, size_t smem);
+int prepare_push(int dim, int prec, int bx, int by, size_t smem);
 int prepare_yee(int dim, int prec, size_t smem);
 int scatter_blocks_per_sm(int dim, int prec);
 
