@@ -48,6 +48,13 @@ static void host_parallel(long long n, long long per_min, F body)
     for (auto& t : th) t.join();
 }
 
+int default_item(long long n, int dim, bool fp64)
+{
+    const long long slots = 152LL * (fp64 ? (dim == 1 ? 2 : 1) : (dim == 3 ? 2 : 4));
+    const long long per = (n + 4 * slots - 1) / (4 * slots);
+    return (int)std::min<long long>(ITEM_MAX, std::max<long long>(256, (per + 255) / 256 * 256));
+}
+
 long long new_group_id()
 {
     static std::atomic<long long> next{1};
@@ -185,7 +192,8 @@ struct Layout {
     int nptiles, nytiles;
     long long cap, max_exits, nslab;
     long long slots;            // slots per particle buffer set: frame factor x cap
-    int chunk, max_chunks;
+    int chunk, max_chunks;      // largest work item; chunks of L.item particles
+    int item;                   // particles per work item of the push (default_item when chunk is 0)
     int tvol, sort_every;       // cells per particle tile; steps between cell sorts (0: none)
     size_t push_smem, yee_smem;
     size_t bytes;
@@ -248,6 +256,19 @@ pic_status validate(const pic_config* c, pic_sim* s)
     return PIC_OK;
 }
 
+long long slab_count(const pic_config* c)
+{
+    long long n = c->ppc > 0 ? c->ppc : 0;
+    for (int d = 0; d < c->dim; ++d) n *= c->slab_hi[d] - c->slab_lo[d];
+    return n;
+}
+
+// particles a simulation can hold
+long long capacity(const pic_config* c)
+{
+    return c->max_particles > 0 ? c->max_particles : std::max<long long>(slab_count(c), 1);
+}
+
 // Tile choice (the autotuner's defaults; `tile` in the config overrides the particle tile).
 void choose_tiles(const pic_config* c, int pt[3], int yt[3])
 {
@@ -256,11 +277,18 @@ void choose_tiles(const pic_config* c, int pt[3], int yt[3])
     if (c->dim == 1) {
         pt[0] = 32; yt[0] = 128;
     } else if (c->dim == 2) {
-        pt[0] = 16; pt[1] = 16; yt[0] = Y2_PX; yt[1] = Y2_PY;
+        // 16x16, or 32x16 where a 16x16 tile of the slab holds less than one default work item
+        // (4.5 M electrons, 4 per cell, items of 2048: push 0.180 -> 0.172 ms; 2.1 M, 8 per cell,
+        // items of 1024: 0.124 with 16x16, 0.127 with 32x16)
+        pt[0] = c->ppc > 0 && 256 * c->ppc < default_item(capacity(c), 2, fp64) ? 32 : 16;
+        pt[1] = 16; yt[0] = Y2_PX; yt[1] = Y2_PY;
     } else {
         // columns of Y3_PX x Y3_PY marching along z in segments: at least ~600 work items
         // (a few per resident block on a full GPU), segments of at most 64 planes
-        pt[0] = 8; pt[1] = 8; pt[2] = 8;
+        // particle tiles: rows of 16 cells in a box of 24 words a row spread the shared-memory
+        // banks; rows of 8 in a box of 16 use half of them (push of 2.0 M electrons at the focus:
+        // 8x8x8 0.469 ms, 8x8x4 0.451, 16x8x4 0.327, 16x4x4 0.328, 32x4x2 0.337)
+        pt[0] = 16; pt[1] = 8; pt[2] = 4;
         yt[0] = Y3_PX; yt[1] = Y3_PY;
         const long long ncol = (long long)ceil_div(c->n[0] + 1, Y3_PX) * ceil_div(c->n[1] + 1, Y3_PY);
         const int nz = c->n[2] + 1;
@@ -313,15 +341,12 @@ Layout make_layout(const pic_config* c)
     L.natot = L.sc;
     L.nptiles = L.npt[0] * L.npt[1] * L.npt[2];
     L.nytiles = L.nyt[0] * L.nyt[1] * L.nyt[2];
-    L.nslab = 0;
-    if (c->ppc > 0) {
-        L.nslab = c->ppc;
-        for (int d = 0; d < c->dim; ++d) L.nslab *= (c->slab_hi[d] - c->slab_lo[d]);
-    }
-    L.cap = c->max_particles > 0 ? c->max_particles : std::max<long long>(L.nslab, 1);
+    L.nslab = slab_count(c);
+    L.cap = capacity(c);
     L.max_exits = c->max_exits > 0 ? c->max_exits : L.cap;
-    L.chunk = c->chunk > 0 ? c->chunk : 2048;
-    L.max_chunks = (int)(L.nptiles + (L.cap + L.chunk - 1) / L.chunk + 1);
+    L.chunk = c->chunk > 0 ? c->chunk : ITEM_MAX;
+    L.item = c->chunk > 0 ? c->chunk : default_item(L.cap, c->dim, c->precision == PIC_FP64);
+    L.max_chunks = (int)(L.nptiles + (L.cap + L.item - 1) / L.item + 1);
     // Every tile keeps slack for the particles within one cell outside it, the only ones a
     // step can bring in (a move is under one cell per axis).  With tiles at least two cells
     // wide a particle lies in the frames of at most 2^dim - 1 other tiles, so 2^dim slots
@@ -655,7 +680,7 @@ pic_status pic_init(const pic_config* cfg_in, const pic_allocator* alloc, void* 
     h.tnum[0] = (int*)A.take((size_t)L.nptiles * 4);
     h.tnum[1] = (int*)A.take((size_t)L.nptiles * 4);
     h.fcnt = (int*)A.take((size_t)L.nptiles * 4);
-    h.chunk = L.chunk;
+    h.chunk = L.item;
     h.lane_p = 8;
     if (cfg->ppc > 0)
         for (h.lane_p = 1; h.lane_p * 2 <= std::min(cfg->ppc, 8);) h.lane_p *= 2;

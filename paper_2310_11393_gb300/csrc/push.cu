@@ -94,16 +94,16 @@ __device__ __forceinline__ R interp(const R* f, const int bx, const int bxy, con
 }
 
 // Current accumulation in the work item's shared-memory box.  FP32: 32-bit fixed point with
-// the scale q = 2^29 / (max(N, 256) w_max) of the item (N particles): a contribution of one
-// particle to one node is bounded by w |v| <= w_max (Esirkepov's partial sums of the shape
+// the scale q = 2^31 (1 - 2^-10) / (max(N, 512) w_max) of the item (N particles): a contribution
+// of one particle to one node is bounded by w |v| <= w_max (Esirkepov's partial sums of the shape
 // change are at most the move in cells, v dt/dx, times dx/dt; the transverse weights are
-// averages of shapes in [0, 1]; |v| < c = 1), so |c q| <= 2^21 and no node's sum leaves
-// 2^29.  Each contribution is rounded to the nearest integer by one FMA with 1.5 * 2^23 (the
-// sum lands in [2^23, 2^24), where the float spacing is 1: its low bits are the rounded
-// integer, exact for |c q| < 2^22) and added with the native shared-memory integer add (the
-// FP32 add is a compare-and-swap loop with a round trip per attempt); zero contributions are
+// averages of shapes in [0, 1]; |v| < c = 1), so |c q| < 2^22 and no node's sum, its N roundings
+// included, reaches 2^31.  Each contribution is rounded to the nearest integer by one FMA with
+// 1.5 * 2^23 (the sum lands in [2^23, 2^24), where the float spacing is 1: its low bits are the
+// rounded integer, exact for |c q| < 2^22) and added with the native shared-memory integer add
+// (the FP32 add is a compare-and-swap loop with a round trip per attempt); zero contributions are
 // added too (no test).  The box is turned back into FP32 before its TMA reduce-add; each
-// contribution's rounding is at most 2^-30 max(N, 256) w_max.  FP64 keeps double sums.
+// contribution's rounding is at most 2^-32 max(N, 512) w_max.  FP64 keeps double sums.
 // Each contribution is a product of a factor c along the current's own axis, scaled by q, and a
 // transverse weight w: the product, its scaling and its rounding are the one FMA.
 __device__ __forceinline__ void jdep(float* a, float c, float w)
@@ -116,7 +116,8 @@ __device__ __forceinline__ void jdep(double* a, double c, double w)
     const double v = c * w;
     if (v != 0.0) atomicAdd(a, v);
 }
-constexpr float JQ_RANGE = 536870912.0f;   // 2^29
+constexpr int JQ_MIN = 512;                        // least N of the scale
+constexpr float JQ_RANGE = 2147483648.0f - 2097152.0f;   // 2^31 (1 - 2^-10)
 
 // Global chunk k of a launch group -> simulation, tile and particle slots.  Chunks are
 // numbered per simulation by the tile scan (ctile / crange) and across the group by gprefix.
@@ -358,7 +359,7 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
         const PhaseRef<R>& pref = s_pref;     // read from shared memory where used (no registers held)
         // fixed-point scale of this item's current (FP32; unused in FP64)
         const float wmax = st->wmax;
-        const R jq = (sizeof(R) == 4 && wmax > 0.f) ? R(JQ_RANGE / ((float)max(p1 - p0, 256) * wmax)) : R(0);
+        const R jq = (sizeof(R) == 4 && wmax > 0.f) ? R(JQ_RANGE / ((float)max(p1 - p0, JQ_MIN) * wmax)) : R(0);
         const R dtdx = bc.dtdx;
         const R jfac = bc.jfac;                     // -q dx/dt, q = -1
         const R hq = bc.hq;                         // q dt / 2
@@ -673,7 +674,7 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
         }
         if constexpr (sizeof(R) == 4) {
             // fixed point back to FP32, in place
-            const float inv = (float)max(p1 - p0, 256) * wmax * (1.0f / JQ_RANGE);
+            const float inv = (float)max(p1 - p0, JQ_MIN) * wmax * (1.0f / JQ_RANGE);
             int* Jq = reinterpret_cast<int*>(Js);
             for (int i = tid; i < 3 * bvol; i += nth) Jq[i] = __float_as_int(__int2float_rn(Jq[i]) * inv);
             __syncthreads();
