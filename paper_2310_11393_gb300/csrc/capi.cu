@@ -681,9 +681,12 @@ pic_status pic_init(const pic_config* cfg_in, const pic_allocator* alloc, void* 
     h.tnum[1] = (int*)A.take((size_t)L.nptiles * 4);
     h.fcnt = (int*)A.take((size_t)L.nptiles * 4);
     h.chunk = L.item;
-    h.lane_p = 8;
-    if (cfg->ppc > 0)
-        for (h.lane_p = 1; h.lane_p * 2 <= std::min(cfg->ppc, 8);) h.lane_p *= 2;
+    h.lane_p = 1;
+    if (L.sort_every > 0) {
+        h.lane_p = 8;
+        if (cfg->ppc > 0)
+            for (h.lane_p = 1; h.lane_p * 2 <= std::min(cfg->ppc, 8);) h.lane_p *= 2;
+    }
     h.max_chunks = L.max_chunks;
     h.tcnt = (int*)A.take((size_t)L.nptiles * 4);
     h.tcur = (int*)A.take((size_t)L.nptiles * 4);
@@ -832,7 +835,7 @@ pic_status pic_init(const pic_config* cfg_in, const pic_allocator* alloc, void* 
         launch_scan_one(s->d, 0, st);
         int hi[3] = {1, 1, 1};
         for (int d = 0; d < cfg->dim; ++d) hi[d] = cfg->slab_hi[d];
-        launch_place_slab(s->d, cfg->dim, cfg->precision, L.nslab, cfg->ppc, lo, hi, st);
+        launch_place_slab(s->d, cfg->dim, cfg->precision, L.nslab, cfg->ppc, lo, hi, L.sort_every > 0, st);
         INIT_CHECK(cudaGetLastError());
     }
     // the first push's destination slots (set 1): tile counts plus frame counts

@@ -365,14 +365,16 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
         const R hq = bc.hq;                         // q dt / 2
         const int hx[3] = {4, 2, 2};                // box halo below the tile per axis
 
-        // Rounds of nth particles (256 or 512).  With P particles per cell (1, 2, 4 or 8) sitting next to
-        // each other after the sort, lane l of warp w takes particle P l + (w mod P) of the
-        // round's (w div P)-th group of 32 P: the 32 lanes of a warp then sit in 32
-        // consecutive cells, so the same stencil node of the deposit and the gather is a
-        // different shared-memory word (mostly a different bank) in every lane.
+        // Rounds of nth particles (256 or 512).  Thread t takes particle t of the round: the
+        // placement below writes a warp's particles into consecutive slots in lane order, so
+        // slots that started as 32 consecutive cells (k_place_slab) stay close to that, whatever
+        // the plasma does, and the loads are coalesced.  With a cell sort the P particles of a
+        // cell (1, 2, 4 or 8) sit next to each other instead: lane l of warp w then takes particle
+        // P l + (w mod P) of the round's (w div P)-th group of 32 P.  Either way a stencil node of
+        // the deposit and the gather is mostly a different shared-memory word in every lane.
         const int P = S.lane_p, wq = tid >> 5;
         int q = (tid & 31) * P + (wq & (P - 1)) + 32 * P * (wq / P);
-        if (S.pt[0] == 16 && P <= 4) {
+        if (S.pt[0] == 16 && P > 1 && P <= 4) {
             // 16-cell tile rows: a warp's 32 cells span two rows.  The box row pitch is 24
             // words, so rows two apart start 16 banks apart: the warp's groups take rows
             // (r, r + 2) of the round instead of (r, r + 1), and its two half-warps hit
@@ -1374,12 +1376,16 @@ __global__ void k_sort_linear(const SimDev* __restrict__ sim, long long n)
     }
 }
 
-// Seeded slab, set 1 (generation order: ppc particles per slab cell, x fastest) -> set 0,
-// placed directly in cell order within each tile: a particle of cell c goes to
+// Seeded slab, set 1 (generation order: ppc particles per slab cell, x fastest) -> set 0.
+// bycell (simulations with a cell sort): in cell order within each tile, a particle of cell c to
 // toff[tile] + (rank of c among the tile's slab cells, x fastest) ppc + (its index in c).
+// Otherwise the first particles of all the tile's cells, then the second ones and so on, each in
+// cell order: 32 consecutive slots hold 32 consecutive cells, one warp of the push.  Where the
+// tile's slab rows are 16 cells long such a warp takes rows r and r + 2 (16 banks apart in the
+// push's box, rows r and r + 1 would overlap): the rows of a plane are numbered 0 2 1 3 4 6 5 7 ...
 template <int D, typename R>
 __global__ void k_place_slab(const SimDev* __restrict__ sim, long long n, int ppc, int lo0, int lo1, int lo2,
-                             int hi0, int hi1, int hi2)
+                             int hi0, int hi1, int hi2, bool bycell)
 {
     const SimDev& S = *sim;
     const int slo[3] = {lo0, lo1, lo2}, shi[3] = {hi0, hi1, hi2};
@@ -1389,14 +1395,19 @@ __global__ void k_place_slab(const SimDev* __restrict__ sim, long long n, int pp
         decode_cell<D>(S, S.cell[1][p], c);
         const int t = tile_of<D>(S, c);
         long long rank = 0, width = 1;
+        long long row0 = 0;
 #pragma unroll
         for (int d = 0; d < D; ++d) {
             const int a = max(slo[d], (c[d] / S.pt[d]) * S.pt[d]);
             const int b = min(shi[d], (c[d] / S.pt[d] + 1) * S.pt[d]);
-            rank += (c[d] - a) * width;
+            int i = c[d] - a;
+            if (d == 0) row0 = b - a;
+            if (d == 1 && !bycell && row0 == 16 && (i | 3) < b - a && ((i & 3) == 1 || (i & 3) == 2)) i ^= 3;
+            rank += i * width;
             width *= (b - a);
         }
-        copy_particle<D, R>(S, 1, p, 0, (long long)S.toff[0][t] + rank * ppc + (p % ppc));
+        copy_particle<D, R>(S, 1, p, 0,
+                            (long long)S.toff[0][t] + (bycell ? rank * ppc + (p % ppc) : (p % ppc) * width + rank));
     }
 }
 
@@ -1540,15 +1551,15 @@ static void sortlin_t(const SimDev* sim, long long n, cudaStream_t s)
     if (n > 0) k_sort_linear<D, R><<<grid, 256, 0, s>>>(sim, n);
 }
 template <int D, typename R>
-static void place_t(const SimDev* sim, long long n, int ppc, const int lo[3], const int hi[3], cudaStream_t s)
+static void place_t(const SimDev* sim, long long n, int ppc, const int lo[3], const int hi[3], bool bycell, cudaStream_t s)
 {
     const int grid = (int)std::min<long long>((n + 255) / 256, (long long)device_sms() * 16);
-    if (n > 0) k_place_slab<D, R><<<grid, 256, 0, s>>>(sim, n, ppc, lo[0], lo[1], lo[2], hi[0], hi[1], hi[2]);
+    if (n > 0) k_place_slab<D, R><<<grid, 256, 0, s>>>(sim, n, ppc, lo[0], lo[1], lo[2], hi[0], hi[1], hi[2], bycell);
 }
 void launch_place_slab(const SimDev* sim, int dim, int prec, long long n, int ppc, const int lo[3], const int hi[3],
-                       cudaStream_t s)
+                       bool bycell, cudaStream_t s)
 {
-    SFF_DISPATCH(dim, prec, place_t, sim, n, ppc, lo, hi, s);
+    SFF_DISPATCH(dim, prec, place_t, sim, n, ppc, lo, hi, bycell, s);
 }
 
 void launch_sort_linear(const SimDev* sim, int dim, int prec, long long n, cudaStream_t s)

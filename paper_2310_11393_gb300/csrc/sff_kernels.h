@@ -80,7 +80,7 @@ void launch_gen_slab(const SimDev* sim, int dim, int prec, long long n, int ppc,
 void launch_count_linear(const SimDev* sim, int dim, int prec, long long n, cudaStream_t s);
 void launch_sort_linear(const SimDev* sim, int dim, int prec, long long n, cudaStream_t s);
 void launch_place_slab(const SimDev* sim, int dim, int prec, long long n, int ppc, const int lo[3], const int hi[3],
-                       cudaStream_t s);
+                       bool bycell, cudaStream_t s);
 // set-up: compact slots of set q from the counts, then (after the particles are placed)
 // the frame counts of its n particles and the slots of set 1 - q
 void launch_scan_one(const SimDev* sim, int q, cudaStream_t s);
