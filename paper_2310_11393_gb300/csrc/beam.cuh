@@ -67,23 +67,22 @@ inline BeamC<R> make_beam_consts(const SimDev& S)
     b.hq = R(-0.5 * S.dt);
     b.dtdx = R(S.dt * S.inv_dx);
     b.jfac = R(S.dx / S.dt);
+    // |w|^{-(s+1)} below e^{-36}: the term is below ~1e-11 of the peak field even after the
+    // largest 1/R^5 and polynomial factors the closed form applies.  The + term is also left out
+    // where it is below e^{-18} (FP32; FP64 e^{-42}) of the - term: a quarter of the rounding
+    // of the - term in every sum the two enter.
+    b.wcut = R(std::exp(72.0 / (S.s + 1.0)));
+    b.wrel = R(std::exp((sizeof(R) == 4 ? 36.0 : 84.0) / (S.s + 1.0)));
+    b.aos = R(S.s > 0 ? S.a / S.s : 0.0);
     return b;
 }
 
-// log|w|, w = 1 - i tau/s (decides whether the term matters at all)
+// |w|^2 - 1, w = 1 - i tau/s
 template <typename R>
-__device__ __forceinline__ R log_abs_w(const BeamC<R>& b, Cx<R> tau)
+__device__ __forceinline__ R w2m1(const BeamC<R>& b, Cx<R> tau)
 {
     const R ti = tau.y * b.inv_s, tr = tau.x * b.inv_s;
-    return R(0.5) * m_log1p(ti * (R(2) + ti) + tr * tr);
-}
-
-// |w|^{-(s+1)} below e^{-36}: the term is below ~1e-11 of the peak field even after the
-// largest 1/R^5 and polynomial factors the closed form applies, so it is dropped
-template <typename R>
-__device__ __forceinline__ bool negligible(const BeamC<R>& b, R lnw)
-{
-    return b.sp1 * lnw > R(36);
+    return ti * (R(2) + ti) + tr * tr;
 }
 
 __device__ __forceinline__ float m_exp_mag(float x) { return __expf(x); }   // error matters only near x = 0
@@ -102,19 +101,20 @@ __device__ __forceinline__ void sincos_phase(float x, float* s, float* c)
 }
 __device__ __forceinline__ void sincos_phase(double x, double* s, double* c) { sincos(x, s, c); }
 
-// e^{i phi0} w^{-(s+1)}, w = 1 - i tau/s, and g^(1), g^(2) (Eq. poisson_dstr), given log|w|
+// e^{i phi0} w^{-(s+1)}, w = 1 - i tau/s, and g^(1), g^(2) (Eq. poisson_dstr), given |w|^2 - 1
+// (Im tau >= 0, so Re w >= 1)
 template <typename R>
-__device__ __forceinline__ void poisson3(const BeamC<R>& b, Cx<R> tau, R lnw, Cx<R>& g0, Cx<R>& g1, Cx<R>& g2)
+__device__ __forceinline__ void poisson3(const BeamC<R>& b, Cx<R> tau, R x, Cx<R>& g0, Cx<R>& g1, Cx<R>& g2)
 {
     const Cx<R> w = {R(1) + tau.y * b.inv_s, -tau.x * b.inv_s};
-    const R th = m_atan2(w.y, w.x);
-    const R mag = m_exp_mag(-b.sp1 * lnw);
+    const R th = m_atan_right(w.y, w.x);
+    const R mag = m_exp_mag(R(-0.5) * b.sp1 * m_log1p(x));
     R sn, cs;
     sincos_phase(b.phi0 - b.sp1 * th, &sn, &cs);
     g0 = {mag * cs, mag * sn};
     // q = i a/(s w)
-    const R den = R(1) / (b.s * (w.x * w.x + w.y * w.y));
-    const Cx<R> q = {b.a * w.y * den, b.a * w.x * den};
+    const R den = b.aos * m_inv(R(1) + x);
+    const Cx<R> q = {w.y * den, w.x * den};
     g1 = b.sp1 * (g0 * q);
     g2 = b.sp2 * (g1 * q);
 }
@@ -125,7 +125,7 @@ __device__ __noinline__ void phi_series(const BeamC<R>& b, Cx<R> u, R trel, Cx<R
 {
     const Cx<R> w0 = {R(1) + b.a * b.inv_s, -trel * b.inv_s};      // 1 - i(trel + i a)/s
     R lnw = R(0.5) * m_log1p((w0.x * w0.x + w0.y * w0.y) - R(1));
-    if (negligible(b, lnw)) {
+    if (b.sp1 * lnw > R(36)) {
         P[0] = P[1] = P[2] = P[3] = Cx<R>{R(0), R(0)};
         return;
     }
@@ -189,17 +189,25 @@ __device__ __forceinline__ void focused_field(const BeamC<R>& b, R xi, R eta, R 
     const R rho2 = xi * xi + eta * eta;
     const Cx<R> u = {rho2 + zeta * zeta - R(1), R(2) * zeta};
     Cx<R> P[4];
-    if (u.x * u.x + u.y * u.y < b.ring2) {
+    const R uu = u.x * u.x + u.y * u.y;
+    if (uu < b.ring2) {
         phi_series(b, u, trel, P);
     } else {
-        Cx<R> Rr = csqrt_(u);
+        // R = sqrt(u) from |u| (no scaling needed: |u| lies between the ring's edge and the box)
+        const R im = m_isqrt(uu), au = uu * im;       // 1/|u|, |u| = |R|^2
+        const R hp = R(0.5) * (au + m_abs(u.x)), ih = m_isqrt(hp);
+        const R big = hp * ih, small = R(0.5) * m_abs(u.y) * ih;
+        Cx<R> Rr = u.x >= R(0) ? Cx<R>{big, small} : Cx<R>{small, big};
+        if (u.y < R(0)) Rr.y = -Rr.y;
         if (Rr.x * zeta + Rr.y < R(0)) Rr = -Rr;      // Re(R conj(zeta + i)) >= 0
-        const Cx<R> den = {Rr.x + zeta, Rr.y + R(1)};
-        const Cx<R> qq = (b.a * rho2) * cinv(den);     // a R - (z + i a)
+        const Cx<R> den = {Rr.x + zeta, Rr.y + R(1)};   // |den| >= |zeta + i| >= 1
+        const R qd = (b.a * rho2) * m_inv(den.x * den.x + den.y * den.y);
+        const Cx<R> qq = {qd * den.x, -qd * den.y};    // a R - (z + i a)
         const Cx<R> taum = {tmz - qq.x, -qq.y};
         const Cx<R> taup = {tpz + qq.x, b.two_a + qq.y};
-        const R lnm = log_abs_w(b, taum), lnp = log_abs_w(b, taup);
-        const bool use_m = !negligible(b, lnm), use_p = !negligible(b, lnp);
+        const R xm = w2m1(b, taum), xp = w2m1(b, taup);
+        const bool use_m = R(1) + xm < b.wcut;
+        const bool use_p = R(1) + xp < b.wcut && R(1) + xp < b.wrel * (R(1) + xm);
         if (!use_m && !use_p) {
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
@@ -208,12 +216,29 @@ __device__ __forceinline__ void focused_field(const BeamC<R>& b, R xi, R eta, R 
             }
             return;
         }
-        Cx<R> g0m = {0, 0}, g1m = {0, 0}, g2m = {0, 0}, g0p = {0, 0}, g1p = {0, 0}, g2p = {0, 0};
-        if (use_m) poisson3(b, taum, lnm, g0m, g1m, g2m);
-        if (use_p) poisson3(b, taup, lnp, g0p, g1p, g2p);
-        const Cx<R> G0m = g0p - g0m, G1p = g1p + g1m, G1m = g1p - g1m, G2p = g2p + g2m, G2m = g2p - g2m;
-        const Cx<R> iR = cinv(Rr);
-        const Cx<R> iR2 = iR * iR;
+        // G^(n)_pm = g^(n)(tau_+) +- g^(n)(tau_-)
+        Cx<R> G0m = {0, 0}, G1p = {0, 0}, G1m = {0, 0}, G2p = {0, 0}, G2m = {0, 0};
+        if (use_m) {
+            Cx<R> g0, g1, g2;
+            poisson3(b, taum, xm, g0, g1, g2);
+            G0m = -g0;
+            G1p = g1;
+            G1m = -g1;
+            G2p = g2;
+            G2m = -g2;
+        }
+        if (use_p) {
+            Cx<R> g0, g1, g2;
+            poisson3(b, taup, xp, g0, g1, g2);
+            G0m = G0m + g0;
+            G1p = G1p + g1;
+            G1m = G1m + g1;
+            G2p = G2p + g2;
+            G2m = G2m + g2;
+        }
+        const Cx<R> iR = {Rr.x * im, -Rr.y * im};
+        const R im2 = im * im;
+        const Cx<R> iR2 = {u.x * im2, -u.y * im2};
         const Cx<R> iR3 = iR2 * iR;
         P[0] = R(0.5) * (G1p * iR2 - G0m * iR3);
         P[1] = R(0.25) * ((G2m * iR3) - R(3) * ((G1p * iR2) * iR2) + R(3) * ((G0m * iR3) * iR2));

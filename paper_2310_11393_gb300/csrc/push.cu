@@ -171,7 +171,7 @@ __device__ __forceinline__ void boris_update(R u[3], const R E[3], const R B[3],
     const R tf = h * m_rsqrt(R(1) + um[0] * um[0] + um[1] * um[1] + um[2] * um[2]);   // h / gamma^-
     const R tv[3] = {tf * B[0], tf * B[1], tf * B[2]};
     const R t2 = tv[0] * tv[0] + tv[1] * tv[1] + tv[2] * tv[2];
-    const R sf = R(2) / (R(1) + t2);
+    const R sf = R(2) * m_inv(R(1) + t2);
     const R up[3] = {um[0] + (um[1] * tv[2] - um[2] * tv[1]), um[1] + (um[2] * tv[0] - um[0] * tv[2]),
                      um[2] + (um[0] * tv[1] - um[1] * tv[0])};
     const R sv[3] = {sf * tv[0], sf * tv[1], sf * tv[2]};
