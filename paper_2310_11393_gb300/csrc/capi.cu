@@ -156,6 +156,21 @@ double s_from_duration_h(int beam, double a, double dur)
 }
 
 int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
+
+// bytes of the tiles' first-record table at the head of the staging memory
+size_t stage_head(int nptiles) { return align256((size_t)(nptiles + 1) * 4); }
+
+// Maps the pages of a host output buffer (one byte written per page, on several threads): a
+// copy into pages that are not mapped yet runs at the rate of one thread's page faults
+// (14-22 GB/s, mapped 190 GB/s).  The caller overwrites every byte.
+void touch_pages(void* p, size_t bytes)
+{
+    const size_t page = 65536;       // the page size of the GPU's host; smaller pages: most faults
+    if (bytes < (1u << 20)) return;
+    host_parallel((long long)(bytes / page), 64, [=](long long a, long long b) {
+        for (long long k = a; k < b; ++k) static_cast<volatile char*>(p)[(size_t)k * page] = 0;
+    });
+}
 int bits_for(int n)
 {
     int b = 0;
@@ -196,6 +211,7 @@ struct Layout {
     int item;                   // particles per work item of the push (default_item when chunk is 0)
     int tvol, sort_every;       // cells per particle tile; steps between cell sorts (0: none)
     size_t push_smem, yee_smem;
+    size_t stage;               // scratch: charge density, staging of state conversions
     size_t bytes;
 };
 
@@ -380,7 +396,11 @@ Layout make_layout(const pic_config* c)
     b += 2 * align256((size_t)L.max_chunks * 4) + 2 * align256((size_t)L.max_chunks * 8);   // ctile, crange
     if (L.sort_every > 0) b += 2 * align256((size_t)tcells * 4);
     b += align256((size_t)L.max_exits * EXIT_DOUBLES * 8);
-    b += 2 * align256((size_t)L.natot * 8);
+    // scratch holds a component of the grid in double, and up to 64 MB of particle records behind
+    // the tiles' first records
+    L.stage = std::max((size_t)L.natot * 8,
+                       stage_head(L.nptiles) + (size_t)std::min<long long>(64 * L.cap, 64ll << 20));
+    b += align256((size_t)L.natot * 8) + align256(L.stage);
     b += align256((size_t)L.nytiles * sizeof(Work));
     b += align256(64) + align256(64) + align256(8 * 8) + align256(8);
     L.bytes = b;
@@ -704,7 +724,8 @@ pic_status pic_init(const pic_config* cfg_in, const pic_allocator* alloc, void* 
     h.scanticket = (int*)A.take(4);
     h.exits = (double*)A.take((size_t)L.max_exits * EXIT_DOUBLES * 8);
     h.rho_ion = (double*)A.take((size_t)L.natot * 8);
-    h.scratch = (double*)A.take((size_t)L.natot * 8);
+    h.scratch = (double*)A.take(L.stage);
+    s->stage_bytes = L.stage;
     s->d_ywork = (Work*)A.take((size_t)L.nytiles * sizeof(Work));
     s->d_gprefix = (int*)A.take(64);
     s->d_counters = (int*)A.take(64);
@@ -1004,67 +1025,32 @@ pic_status pic_set_particles(pic_sim* s, int64_t n, const double* x, const doubl
                                           (long long)s->pcap);
     if (n > 0 && (!x || !u || !w || !id)) return fail(s, PIC_EINVAL, "NULL particle array");
     cudaStream_t st = (cudaStream_t)stream;
-    const int D = s->cfg.dim, es = s->es;
-    // host copies in the device layout (left uninitialised: every byte is written below)
-    std::unique_ptr<unsigned[]> cell(new unsigned[n > 0 ? n : 1]), pid(new unsigned[n > 0 ? n : 1]);
-    std::unique_ptr<char[]> off(new char[(size_t)D * n * es + 1]), mom(new char[(size_t)3 * n * es + 1]),
-        wt(new char[(size_t)n * es + 1]);
-    // converted on several host threads; each range reports its first invalid particle
-    const int nb = 16;
-    std::vector<long long> bad(nb, -1);
-    std::vector<double> wmx(nb, 0.0);       // largest |weight| of each range
-    std::atomic<int> slot{0}, wslot{0};
-    host_parallel(n, 1 << 16, [&](long long p0, long long p1) {
-        long long first = -1;
-        double wm_r = 0.0;
-        for (long long p = p0; p < p1 && first < 0; ++p) {
-            wm_r = std::max(wm_r, std::fabs(w[p]));
-            int c[3] = {0, 0, 0};
-            for (int d = 0; d < D; ++d) {
-                const double X = x[3 * p + d] / s->cfg.dx;
-                const double fl = std::floor(X);
-                c[d] = (int)fl;
-                if (!(X >= s->h.margin) || !(X < s->h.n[d] - s->h.margin)) first = p;
-                double o = X - fl;
-                if (es == 4) {
-                    float of = (float)o;
-                    if (of >= 1.0f) of = std::nextafter(1.0f, 0.0f);
-                    memcpy(&off[((size_t)d * n + p) * 4], &of, 4);
-                } else {
-                    memcpy(&off[((size_t)d * n + p) * 8], &o, 8);
-                }
-            }
-            if (id[p] < 0 || id[p] >= (1ll << 31)) first = p;
-            unsigned v = (unsigned)c[0];
-            if (D > 1) v |= (unsigned)c[1] << s->h.cb[0];
-            if (D > 2) v |= (unsigned)c[2] << (s->h.cb[0] + s->h.cb[1]);
-            cell[p] = v;
-            pid[p] = (unsigned)id[p];
-            for (int d = 0; d < 3; ++d) {
-                if (es == 4) {
-                    float f = (float)u[3 * p + d];
-                    memcpy(&mom[((size_t)d * n + p) * 4], &f, 4);
-                } else {
-                    memcpy(&mom[((size_t)d * n + p) * 8], &u[3 * p + d], 8);
-                }
-            }
-            if (es == 4) {
-                float f = (float)w[p];
-                memcpy(&wt[(size_t)p * 4], &f, 4);
-            } else {
-                memcpy(&wt[(size_t)p * 8], &w[p], 8);
-            }
-        }
-        if (first >= 0) {
-            const int k = slot.fetch_add(1);
-            if (k < nb) bad[k] = first;
-        }
-        const int kw = wslot.fetch_add(1);
-        if (kw < nb) wmx[kw] = wm_r;
-    });
-    long long first_bad = -1;
-    for (long long b : bad)
-        if (b >= 0 && (first_bad < 0 || b < first_bad)) first_bad = b;
+    const int D = s->cfg.dim;
+    // pieces that fit the staging memory: x, u, w, id of up to `piece` particles
+    const long long piece = std::max<long long>(1, std::min<long long>(n, (long long)(s->stage_bytes / 64)));
+    double* sx = s->h.scratch;
+    double *su = sx + 3 * piece, *sw = su + 3 * piece;
+    long long* sid = reinterpret_cast<long long*>(sw + piece);
+    auto load = [&](long long k0, int m, bool all) -> cudaError_t {
+        cudaError_t e = cudaMemcpyAsync(sx, x + 3 * k0, (size_t)m * 24, cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess && all) e = cudaMemcpyAsync(su, u + 3 * k0, (size_t)m * 24, cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(sw, w + k0, (size_t)m * 8, cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(sid, id + k0, (size_t)m * 8, cudaMemcpyHostToDevice, st);
+        return e;
+    };
+    // first pass: nothing of the simulation changes unless every particle is accepted
+    unsigned long long chk[2] = {~0ull, 0ull};
+    unsigned long long* d_chk = reinterpret_cast<unsigned long long*>(s->d_acc);
+    CU_CHECK(s, cudaMemcpyAsync(d_chk, chk, sizeof chk, cudaMemcpyHostToDevice, st));
+    for (long long k0 = 0; k0 < n; k0 += piece) {
+        const int m = (int)std::min<long long>(piece, n - k0);
+        CU_CHECK(s, load(k0, m, n <= piece));
+        launch_check_particles(s->d, D, k0, m, sx, sw, sid, d_chk, st);
+        CU_CHECK(s, cudaGetLastError());
+    }
+    CU_CHECK(s, cudaMemcpyAsync(chk, d_chk, sizeof chk, cudaMemcpyDeviceToHost, st));
+    CU_CHECK(s, cudaStreamSynchronize(st));
+    const long long first_bad = chk[0] == ~0ull ? -1 : (long long)chk[0];
     if (first_bad >= 0) {
         const long long p = first_bad;
         if (id[p] < 0 || id[p] >= (1ll << 31)) {
@@ -1082,16 +1068,11 @@ pic_status pic_set_particles(pic_sim* s, int64_t n, const double* x, const doubl
         }
         return fail(s, PIC_EINVAL, "particle id out of range");
     }
-    if (n > 0) {
-        CU_CHECK(s, cudaMemcpyAsync(s->h.cell[1], cell.get(), n * 4, cudaMemcpyHostToDevice, st));
-        CU_CHECK(s, cudaMemcpyAsync(s->h.pid[1], pid.get(), n * 4, cudaMemcpyHostToDevice, st));
-        for (int d = 0; d < D; ++d)
-            CU_CHECK(s, cudaMemcpyAsync(s->h.off[1][d], &off[(size_t)d * n * es], n * es, cudaMemcpyHostToDevice, st));
-        for (int d = 0; d < 3; ++d)
-            CU_CHECK(s, cudaMemcpyAsync(s->h.mom[1][d], &mom[(size_t)d * n * es], n * es, cudaMemcpyHostToDevice, st));
-        CU_CHECK(s, cudaMemcpyAsync(s->h.wgt[1], wt.get(), n * es, cudaMemcpyHostToDevice, st));
-        // the host copies are released on return: the copies must have read them
-        CU_CHECK(s, cudaStreamSynchronize(st));
+    for (long long k0 = 0; k0 < n; k0 += piece) {
+        const int m = (int)std::min<long long>(piece, n - k0);
+        if (n > piece) CU_CHECK(s, load(k0, m, true));
+        launch_put_particles(s->d, D, s->cfg.precision, k0, m, sx, su, sw, sid, st);
+        CU_CHECK(s, cudaGetLastError());
     }
     s->prefix_group = 0;   // a new layout: the next step numbers its chunks first
     pic_status r = sort_linear_into_set0(s, n, st);
@@ -1101,8 +1082,8 @@ pic_status pic_set_particles(pic_sim* s, int64_t n, const double* x, const doubl
     if ((r = read_state(s, &ds, st)) != PIC_OK) return r;
     {
         // largest |weight| (rounded up in FP32): the scale of the FP32 push's fixed-point current
-        double wm = 0.0;
-        for (double v : wmx) wm = std::max(wm, v);
+        double wm;
+        memcpy(&wm, &chk[1], 8);
         ds.wmax = wm > 0 ? std::nextafter((float)wm, INFINITY) : 0.f;
         if ((r = write_state(s, ds, st)) != PIC_OK) return r;
     }
@@ -1118,45 +1099,12 @@ pic_status pic_set_fields(pic_sim* s, const double* fields, void* stream)
     pic_status r = read_state(s, &ds, st);
     if (r != PIC_OK) return r;
     const int D = s->cfg.dim;
-    const int ext[3] = {s->h.n[0] + 1, D > 1 ? s->h.n[1] + 1 : 1, D > 2 ? s->h.n[2] + 1 : 1};
-    const long long ne = (long long)ext[0] * ext[1] * ext[2];
-    // the device layout of E, B (zero at the points a component does not have and in the
-    // ghost region), zero-filled on several host threads
-    const size_t nbuf = (size_t)6 * s->nalloc_tot * s->es;
-    std::unique_ptr<char[]> buf(new char[nbuf]);
-    host_parallel((long long)((nbuf + 4095) / 4096), 1 << 10, [&](long long b0, long long b1) {
-        const size_t a = (size_t)b0 * 4096, e = std::min(nbuf, (size_t)b1 * 4096);
-        memset(buf.get() + a, 0, e - a);
-    });
-    // rows (comp, k, j) of the host array converted on up to 16 host threads
-    const long long nrows = 6LL * ext[2] * ext[1];
-    host_parallel(nrows, 256, [&](long long r0, long long r1) {
-        for (long long r = r0; r < r1; ++r) {
-            const int j = (int)(r % ext[1]), k = (int)((r / ext[1]) % ext[2]), comp = (int)(r / ((long long)ext[1] * ext[2]));
-            const int c = comp % 3;
-            for (int i = 0; i < ext[0]; ++i) {
-                const int g[3] = {i, j, k};
-                bool has = true;
-                for (int d = 0; d < D; ++d) {
-                    const bool stag = comp < 3 ? (d == c) : (d != c);
-                    if (stag && g[d] > s->h.n[d] - 1) has = false;
-                }
-                if (!has) continue;
-                const double v = fields[comp * ne + ((long long)k * ext[1] + j) * ext[0] + i];
-                const long long o = comp * s->nalloc_tot + (long long)(D > 2 ? k + G : 0) * s->h.sz +
-                                    (long long)(D > 1 ? j + G : 0) * s->h.sy + (i + GX);
-                if (s->es == 4) {
-                    float f = (float)v;
-                    memcpy(&buf[o * 4], &f, 4);
-                } else {
-                    memcpy(&buf[o * 8], &v, 8);
-                }
-            }
-        }
-    });
-    char* F = (char*)s->h.F;
-    CU_CHECK(s, cudaMemcpyAsync(F + (size_t)comp_eb(ds.parity) * s->nalloc_tot * s->es, buf.get(), nbuf,
-                                cudaMemcpyHostToDevice, st));
+    const long long ne = (long long)(s->h.n[0] + 1) * (D > 1 ? s->h.n[1] + 1 : 1) * (D > 2 ? s->h.n[2] + 1 : 1);
+    for (int comp = 0; comp < 6; ++comp) {
+        CU_CHECK(s, cudaMemcpyAsync(s->h.scratch, fields + comp * ne, (size_t)ne * 8, cudaMemcpyHostToDevice, st));
+        launch_put_field(s->d, D, s->cfg.precision, s->nalloc_tot, comp_eb(ds.parity) + comp, comp, s->h.scratch, st);
+        CU_CHECK(s, cudaGetLastError());
+    }
     CU_CHECK(s, cudaStreamSynchronize(st));
     return PIC_OK;
 }
@@ -1213,66 +1161,25 @@ pic_status pic_diag(pic_sim* s, int kind, void* host_out, size_t bytes, void* st
     case PIC_DIAG_PARTICLES: {
         const long long n = ds.n_alive;
         if (bytes < (size_t)n * 8 * sizeof(double)) return fail(s, PIC_ECAPACITY, "PARTICLES needs %lld bytes", n * 64);
-        const int q = ds.parity, es = s->es, nt = s->h.nptiles;
+        const int q = ds.parity, nt = s->h.nptiles;
         // the tiles' occupied slots of the current set, in tile order
-        std::vector<int> toff(nt + 1), tnum(nt);
-        CU_CHECK(s, cudaMemcpyAsync(toff.data(), s->h.toff[q], (nt + 1) * 4, cudaMemcpyDeviceToHost, st));
-        CU_CHECK(s, cudaMemcpyAsync(tnum.data(), s->h.tnum[q], nt * 4, cudaMemcpyDeviceToHost, st));
+        int* first = reinterpret_cast<int*>(s->h.scratch);
+        double* rec = s->h.scratch + stage_head(nt) / 8;
+        const long long piece = std::max<long long>(1, (long long)((s->stage_bytes - stage_head(nt)) / 64));
+        int tot = 0;
+        launch_tile_first(s->d, q, first, st);
+        CU_CHECK(s, cudaMemcpyAsync(&tot, first + nt, 4, cudaMemcpyDeviceToHost, st));
         CU_CHECK(s, cudaStreamSynchronize(st));
-        const long long nu = std::min<long long>(toff[nt], s->h.cap);
-        long long tot = 0;
-        for (int t = 0; t < nt; ++t) tot += tnum[t];
-        if (tot != n) return fail(s, PIC_ECUDA, "tile counts (%lld) disagree with the particle count (%lld)", tot, n);
-        // host copies (left uninitialised: the copies fill them)
-        std::unique_ptr<unsigned[]> cell(new unsigned[nu + 1]), pid(new unsigned[nu + 1]);
-        std::unique_ptr<char[]> off(new char[(size_t)D * nu * es + 1]), mom(new char[(size_t)3 * nu * es + 1]),
-            wt(new char[(size_t)nu * es + 1]);
-        if (nu > 0) {
-            CU_CHECK(s, cudaMemcpyAsync(cell.get(), s->h.cell[q], nu * 4, cudaMemcpyDeviceToHost, st));
-            CU_CHECK(s, cudaMemcpyAsync(pid.get(), s->h.pid[q], nu * 4, cudaMemcpyDeviceToHost, st));
-            for (int d = 0; d < D; ++d)
-                CU_CHECK(s, cudaMemcpyAsync(&off[(size_t)d * nu * es], s->h.off[q][d], nu * es, cudaMemcpyDeviceToHost, st));
-            for (int d = 0; d < 3; ++d)
-                CU_CHECK(s, cudaMemcpyAsync(&mom[(size_t)d * nu * es], s->h.mom[q][d], nu * es, cudaMemcpyDeviceToHost, st));
-            CU_CHECK(s, cudaMemcpyAsync(wt.get(), s->h.wgt[q], nu * es, cudaMemcpyDeviceToHost, st));
+        if (tot != n) return fail(s, PIC_ECUDA, "tile counts (%d) disagree with the particle count (%lld)", tot, n);
+        for (long long k0 = 0; k0 < n; k0 += piece) {
+            const long long k1 = std::min(n, k0 + piece);
+            launch_pack_particles(s->d, D, s->cfg.precision, q, nt, first, k0, k1, rec, st);
+            CU_CHECK(s, cudaGetLastError());
+            char* dst = (char*)host_out + (size_t)k0 * 64;
+            touch_pages(dst, (size_t)(k1 - k0) * 64);
+            CU_CHECK(s, cudaMemcpyAsync(dst, rec, (size_t)(k1 - k0) * 64, cudaMemcpyDeviceToHost, st));
         }
         CU_CHECK(s, cudaStreamSynchronize(st));
-        auto rd = [&](const char* v, size_t idx) {
-            if (es == 4) {
-                float f;
-                memcpy(&f, v + idx * 4, 4);
-                return (double)f;
-            }
-            double xv;
-            memcpy(&xv, v + idx * 8, 8);
-            return xv;
-        };
-        // record k of the output = the tiles' particles in tile order; tiles converted on
-        // several host threads from their first record index
-        std::vector<long long> first(nt + 1, 0);
-        for (int t = 0; t < nt; ++t)
-            first[t + 1] = first[t] + std::max<long long>(0, std::min<long long>((long long)toff[t] + tnum[t], nu) - toff[t]);
-        if (first[nt] != n) return fail(s, PIC_ECUDA, "tile slots hold %lld particles, expected %lld", first[nt], n);
-        double* o = (double*)host_out;
-        host_parallel(nt, std::max<long long>(1, (1 << 16) * (long long)nt / std::max<long long>(n, 1)),
-                      [&](long long t0, long long t1) {
-            for (long long t = t0; t < t1; ++t) {
-                long long k = first[t];
-                const long long p1 = std::min<long long>((long long)toff[t] + tnum[t], nu);
-                for (long long p = toff[t]; p < p1; ++p, ++k) {
-                    const unsigned cl = cell[p];
-                    int c[3];
-                    c[0] = (int)(cl & ((1u << s->h.cb[0]) - 1u));
-                    c[1] = D > 1 ? (int)((cl >> s->h.cb[0]) & ((1u << s->h.cb[1]) - 1u)) : 0;
-                    c[2] = D > 2 ? (int)(cl >> (s->h.cb[0] + s->h.cb[1])) : 0;
-                    for (int d = 0; d < 3; ++d)
-                        o[8 * k + d] = d < D ? ((double)c[d] + rd(off.get(), (size_t)d * nu + p)) * s->cfg.dx : 0.0;
-                    for (int d = 0; d < 3; ++d) o[8 * k + 3 + d] = rd(mom.get(), (size_t)d * nu + p);
-                    o[8 * k + 6] = rd(wt.get(), p);
-                    o[8 * k + 7] = (double)pid[p];
-                }
-            }
-        });
         return PIC_OK;
     }
     case PIC_DIAG_EXITS: {
@@ -1286,48 +1193,16 @@ pic_status pic_diag(pic_sim* s, int kind, void* host_out, size_t bytes, void* st
         const int ext[3] = {s->h.n[0] + 1, D > 1 ? s->h.n[1] + 1 : 1, D > 2 ? s->h.n[2] + 1 : 1};
         const long long ne = (long long)ext[0] * ext[1] * ext[2];
         if (bytes < (size_t)9 * ne * 8) return fail(s, PIC_ECAPACITY, "FIELDS needs %lld bytes", 9 * ne * 8);
-        const int es = s->es;
-        std::vector<char> eb((size_t)6 * s->nalloc_tot * es), jb((size_t)3 * s->nalloc_tot * es);
-        const char* F = (const char*)s->h.F;
-        CU_CHECK(s, cudaMemcpyAsync(eb.data(), F + (size_t)comp_eb(ds.parity) * s->nalloc_tot * es, eb.size(),
-                                    cudaMemcpyDeviceToHost, st));
-        // the current deposited by the last step sits in J of the other set
-        CU_CHECK(s, cudaMemcpyAsync(jb.data(), F + (size_t)comp_j(1 - ds.parity) * s->nalloc_tot * es, jb.size(),
-                                    cudaMemcpyDeviceToHost, st));
-        CU_CHECK(s, cudaStreamSynchronize(st));
         double* o = (double*)host_out;
-        // rows (comp, k, j) of the host array converted on up to 16 host threads
-        const long long nrows = 9LL * ext[2] * ext[1];
-        host_parallel(nrows, 256, [&](long long r0, long long r1) {
-            for (long long r = r0; r < r1; ++r) {
-                const int j = (int)(r % ext[1]), k = (int)((r / ext[1]) % ext[2]);
-                const int comp = (int)(r / ((long long)ext[1] * ext[2]));
-                const std::vector<char>& src = comp < 6 ? eb : jb;
-                const int sc = comp < 6 ? comp : comp - 6;
-                const int c = comp % 3;
-                for (int i = 0; i < ext[0]; ++i) {
-                    const int g[3] = {i, j, k};
-                    bool has = true;
-                    for (int d = 0; d < D; ++d) {
-                        const bool stag = (comp < 3 || comp >= 6) ? (d == c) : (d != c);
-                        if (stag && g[d] > s->h.n[d] - 1) has = false;
-                    }
-                    double v = 0.0;
-                    if (has) {
-                        const long long idx = sc * s->nalloc_tot + (long long)(D > 2 ? k + G : 0) * s->h.sz +
-                                              (long long)(D > 1 ? j + G : 0) * s->h.sy + (i + GX);
-                        if (es == 4) {
-                            float f;
-                            memcpy(&f, &src[idx * 4], 4);
-                            v = f;
-                        } else {
-                            memcpy(&v, &src[idx * 8], 8);
-                        }
-                    }
-                    o[comp * ne + ((long long)k * ext[1] + j) * ext[0] + i] = v;
-                }
-            }
-        });
+        for (int comp = 0; comp < 9; ++comp) {
+            // the current deposited by the last step sits in J of the other set
+            const int fc = comp < 6 ? comp_eb(ds.parity) + comp : comp_j(1 - ds.parity) + comp - 6;
+            launch_get_field(s->d, D, s->cfg.precision, ne, fc, comp, s->h.scratch, st);
+            CU_CHECK(s, cudaGetLastError());
+            touch_pages(o + comp * ne, (size_t)ne * 8);
+            CU_CHECK(s, cudaMemcpyAsync(o + comp * ne, s->h.scratch, (size_t)ne * 8, cudaMemcpyDeviceToHost, st));
+        }
+        CU_CHECK(s, cudaStreamSynchronize(st));
         return PIC_OK;
     }
     default:

@@ -265,6 +265,181 @@ __global__ void k_eval_incident(const SimDev* __restrict__ sim, long long n, con
     }
 }
 
+// ---- state to and from the host layout ----------------------------------------------------
+// The conversions between the device layout and the host arrays of the C-ABI run here, one
+// piece of staging memory at a time, and the copy engine moves host doubles: 64 B per electron
+// and 72 B per grid point at the link's rate (190-200 GB/s to and from host pages that are mapped
+// already) instead of a pass of host threads over freshly mapped buffers.  Read-back of 2.1 M
+// electrons 15-22 -> 1.5 ms, of 12 small simulations 21 -> 3 ms.
+
+// first[t]: particles of the tiles before t in buffer set par, first[nptiles] their total
+__global__ void __launch_bounds__(1024) k_tile_first(const SimDev* __restrict__ sim, int par, int* __restrict__ first)
+{
+    const SimDev& S = *sim;
+    __shared__ int s_warp[32];
+    const int tid = threadIdx.x, lane = tid & 31, n = S.nptiles;
+    int carry = 0;
+    for (int base = 0; base < n; base += 1024) {
+        const int i = base + tid;
+        const int v = i < n ? S.tnum[par][i] : 0;
+        int x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) s_warp[tid >> 5] = x;
+        __syncthreads();
+        int before = 0, all = 0;
+        for (int w = 0; w < 32; ++w) {
+            if (w < (tid >> 5)) before += s_warp[w];
+            all += s_warp[w];
+        }
+        if (i < n) first[i] = carry + before + x - v;
+        carry += all;
+        __syncthreads();
+    }
+    if (tid == 0) first[n] = carry;
+}
+
+// records k in [k0, k1) of PIC_DIAG_PARTICLES (tiles in order): x[3], u[3], w, id
+template <int D, typename R>
+__global__ void __launch_bounds__(128) k_pack_particles(const SimDev* __restrict__ sim, int par,
+                                                        const int* __restrict__ first, long long k0, long long k1,
+                                                        double2* __restrict__ out)
+{
+    const SimDev& S = *sim;
+    for (int t = blockIdx.x; t < S.nptiles; t += gridDim.x) {
+        const long long f = first[t], base = S.toff[par][t];
+        const int i0 = (int)max(0ll, k0 - f), i1 = (int)min((long long)S.tnum[par][t], k1 - f);
+        for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
+            const long long p = base + i;
+            int c[3];
+            decode_cell_d<D>(S, S.cell[par][p], c);
+            double r[8] = {0., 0., 0., 0., 0., 0., 0., 0.};
+#pragma unroll
+            for (int d = 0; d < D; ++d) r[d] = ((double)c[d] + (double)reinterpret_cast<const R*>(S.off[par][d])[p]) * S.dx;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) r[3 + d] = (double)reinterpret_cast<const R*>(S.mom[par][d])[p];
+            r[6] = (double)reinterpret_cast<const R*>(S.wgt[par])[p];
+            r[7] = (double)S.pid[par][p];
+            double2* o = out + 4 * (f + i - k0);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) o[j] = make_double2(r[2 * j], r[2 * j + 1]);
+        }
+    }
+}
+
+// largest |w| (ordered bits) and first particle that pic_set_particles refuses: a coordinate
+// outside [margin, n - margin) cells, an id outside [0, 2^31); x, w, id hold particles k0 ..
+template <int D>
+__global__ void k_check_particles(const SimDev* __restrict__ sim, long long k0, int n, const double* __restrict__ x,
+                                  const double* __restrict__ w, const long long* __restrict__ id,
+                                  unsigned long long* __restrict__ out)
+{
+    const SimDev& S = *sim;
+    double wm = 0.0;
+    unsigned long long bad = ~0ull;
+    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
+        bool ok = id[p] >= 0 && id[p] < (1ll << 31);
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+            const double X = x[3 * p + d] / S.dx;
+            ok = ok && X >= S.margin && X < S.n[d] - S.margin;
+        }
+        if (!ok) bad = min(bad, (unsigned long long)(k0 + p));
+        wm = fmax(wm, fabs(w[p]));
+    }
+    unsigned long long wb = (unsigned long long)__double_as_longlong(wm);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        bad = min(bad, __shfl_xor_sync(0xffffffffu, bad, o));
+        wb = max(wb, __shfl_xor_sync(0xffffffffu, wb, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        if (bad != ~0ull) atomicMin(&out[0], bad);
+        atomicMax(&out[1], wb);
+    }
+}
+
+// particles k0 .. k0 + n - 1 from host layout into buffer set 1, linear order
+template <int D, typename R>
+__global__ void k_put_particles(const SimDev* __restrict__ sim, long long k0, int n, const double* __restrict__ x,
+                                const double* __restrict__ u, const double* __restrict__ w,
+                                const long long* __restrict__ id)
+{
+    const SimDev& S = *sim;
+    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
+        unsigned cl = 0;
+        int sh = 0;
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+            const double X = x[3 * p + d] / S.dx;
+            const double fl = floor(X);
+            R o = R(X - fl);
+            if (sizeof(R) == 4 && o >= R(1)) o = R(0.99999994f);      // the float below 1
+            reinterpret_cast<R*>(S.off[1][d])[k0 + p] = o;
+            cl |= (unsigned)(int)fl << sh;
+            sh += S.cb[d];
+        }
+        S.cell[1][k0 + p] = cl;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) reinterpret_cast<R*>(S.mom[1][d])[k0 + p] = R(u[3 * p + d]);
+        reinterpret_cast<R*>(S.wgt[1])[k0 + p] = R(w[p]);
+        S.pid[1][k0 + p] = (unsigned)id[p];
+    }
+}
+
+// is there a point of component comp (0..5 E, B; 6..8 J) at grid index g?
+template <int D>
+__device__ __forceinline__ bool comp_has(const SimDev& S, int comp, const int g[3])
+{
+    const int c = comp % 3;
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+        const bool stag = (comp < 3 || comp >= 6) ? d == c : d != c;
+        if (g[d] < 0 || g[d] > S.n[d] - (stag ? 1 : 0)) return false;
+    }
+    return true;
+}
+
+// component comp of the field array at set offset fc (components) -> out[ext_z][ext_y][ext_x],
+// absent points 0
+template <int D, typename R>
+__global__ void k_get_field(const SimDev* __restrict__ sim, int fc, int comp, double* __restrict__ out)
+{
+    const SimDev& S = *sim;
+    const R* F = reinterpret_cast<const R*>(S.F) + (long long)fc * S.sc;
+    const unsigned ex = S.n[0] + 1, ey = D > 1 ? S.n[1] + 1 : 1, ez = D > 2 ? S.n[2] + 1 : 1;
+    const unsigned rows = ey * ez, bpr = (ex + blockDim.x - 1) / blockDim.x;
+    for (unsigned b = blockIdx.x; b < rows * bpr; b += gridDim.x) {
+        const unsigned r = b / bpr, i = (b - r * bpr) * blockDim.x + threadIdx.x;
+        if (i >= ex) continue;
+        const int g[3] = {(int)i, (int)(r % ey), (int)(r / ey)};
+        const long long o = (long long)(D > 2 ? g[2] + G : 0) * S.sz + (long long)(D > 1 ? g[1] + G : 0) * S.sy + (g[0] + GX);
+        out[(long long)r * ex + i] = comp_has<D>(S, comp, g) ? (double)F[o] : 0.0;
+    }
+}
+
+// in[ext_z][ext_y][ext_x] -> component comp of the field array at offset fc, every allocated
+// point written (zero in the ghost region and at absent points)
+template <int D, typename R>
+__global__ void k_put_field(const SimDev* __restrict__ sim, int fc, int comp, const double* __restrict__ in)
+{
+    const SimDev& S = *sim;
+    R* F = reinterpret_cast<R*>(S.F) + (long long)fc * S.sc;
+    const unsigned ex = S.n[0] + 1, ey = D > 1 ? S.n[1] + 1 : 1;
+    const unsigned nx = S.na[0], ny = S.na[1], rows = ny * (unsigned)S.na[2], bpr = (nx + blockDim.x - 1) / blockDim.x;
+    for (unsigned b = blockIdx.x; b < rows * bpr; b += gridDim.x) {
+        const unsigned r = b / bpr, i = (b - r * bpr) * blockDim.x + threadIdx.x;
+        if (i >= nx) continue;
+        const int g[3] = {(int)i - GX, D > 1 ? (int)(r % ny) - G : 0, D > 2 ? (int)(r / ny) - G : 0};
+        R v = R(0);
+        if (comp_has<D>(S, comp, g)) v = R(in[((long long)g[2] * ey + g[1]) * ex + g[0]]);
+        F[(long long)r * nx + i] = v;
+    }
+}
+
 // ---- host wrappers ----
 static int grid_for(long long n) { return (int)std::max<long long>(1, std::min<long long>((n + 255) / 256, (long long)device_sms() * 8)); }
 
@@ -348,6 +523,66 @@ void launch_eval_incident(const SimDev* sim, int dim, int prec, long long n, con
                           cudaStream_t s)
 {
     SFF_DISPATCH3(dim, prec, evalinc_t, sim, n, pts, out, s);
+}
+
+void launch_tile_first(const SimDev* sim, int par, int* first, cudaStream_t s)
+{
+    k_tile_first<<<1, 1024, 0, s>>>(sim, par, first);
+}
+
+template <int D, typename R>
+static void pack_t(const SimDev* sim, int par, int nptiles, const int* first, long long k0, long long k1, double* out,
+                   cudaStream_t s)
+{
+    const int grid = std::max(1, std::min(nptiles, device_sms() * 16));
+    k_pack_particles<D, R><<<grid, 128, 0, s>>>(sim, par, first, k0, k1, reinterpret_cast<double2*>(out));
+}
+void launch_pack_particles(const SimDev* sim, int dim, int prec, int par, int nptiles, const int* first, long long k0,
+                           long long k1, double* out, cudaStream_t s)
+{
+    SFF_DISPATCH3(dim, prec, pack_t, sim, par, nptiles, first, k0, k1, out, s);
+}
+
+void launch_check_particles(const SimDev* sim, int dim, long long k0, int n, const double* x, const double* w,
+                            const long long* id, unsigned long long* out, cudaStream_t s)
+{
+    if (n <= 0) return;
+    if (dim == 1) k_check_particles<1><<<grid_for(n), 256, 0, s>>>(sim, k0, n, x, w, id, out);
+    else if (dim == 2) k_check_particles<2><<<grid_for(n), 256, 0, s>>>(sim, k0, n, x, w, id, out);
+    else k_check_particles<3><<<grid_for(n), 256, 0, s>>>(sim, k0, n, x, w, id, out);
+}
+
+template <int D, typename R>
+static void put_t(const SimDev* sim, long long k0, int n, const double* x, const double* u, const double* w,
+                  const long long* id, cudaStream_t s)
+{
+    if (n > 0) k_put_particles<D, R><<<grid_for(n), 256, 0, s>>>(sim, k0, n, x, u, w, id);
+}
+void launch_put_particles(const SimDev* sim, int dim, int prec, long long k0, int n, const double* x, const double* u,
+                          const double* w, const long long* id, cudaStream_t s)
+{
+    SFF_DISPATCH3(dim, prec, put_t, sim, k0, n, x, u, w, id, s);
+}
+
+template <int D, typename R>
+static void getf_t(const SimDev* sim, long long points, int fc, int comp, double* out, cudaStream_t s)
+{
+    k_get_field<D, R><<<grid_for(points), 256, 0, s>>>(sim, fc, comp, out);
+}
+void launch_get_field(const SimDev* sim, int dim, int prec, long long points, int fc, int comp, double* out,
+                      cudaStream_t s)
+{
+    SFF_DISPATCH3(dim, prec, getf_t, sim, points, fc, comp, out, s);
+}
+template <int D, typename R>
+static void putf_t(const SimDev* sim, long long points, int fc, int comp, const double* in, cudaStream_t s)
+{
+    k_put_field<D, R><<<grid_for(points), 256, 0, s>>>(sim, fc, comp, in);
+}
+void launch_put_field(const SimDev* sim, int dim, int prec, long long points, int fc, int comp, const double* in,
+                      cudaStream_t s)
+{
+    SFF_DISPATCH3(dim, prec, putf_t, sim, points, fc, comp, in, s);
 }
 
 }  // namespace sff

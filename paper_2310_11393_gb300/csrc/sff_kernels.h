@@ -100,6 +100,23 @@ void launch_histogram(const SimDev* sim, int dim, int prec, long long n_alive, l
 void launch_eval_incident(const SimDev* sim, int dim, int prec, long long n, const double* pts, double* out,
                           cudaStream_t s);
 
+// state to and from the host layout, a piece of staging memory at a time (device pointers):
+// first[nptiles + 1] of the tiles of set par; records [k0, k1) of PIC_DIAG_PARTICLES; the check
+// and the conversion of particles k0 .. k0 + n - 1 (out: first refused index, largest |w| as
+// ordered bits); one field component at offset fc of the field array (points: of the grid, for
+// the launch size)
+void launch_tile_first(const SimDev* sim, int par, int* first, cudaStream_t s);
+void launch_pack_particles(const SimDev* sim, int dim, int prec, int par, int nptiles, const int* first, long long k0,
+                           long long k1, double* out, cudaStream_t s);
+void launch_check_particles(const SimDev* sim, int dim, long long k0, int n, const double* x, const double* w,
+                            const long long* id, unsigned long long* out, cudaStream_t s);
+void launch_put_particles(const SimDev* sim, int dim, int prec, long long k0, int n, const double* x, const double* u,
+                          const double* w, const long long* id, cudaStream_t s);
+void launch_get_field(const SimDev* sim, int dim, int prec, long long points, int fc, int comp, double* out,
+                      cudaStream_t s);
+void launch_put_field(const SimDev* sim, int dim, int prec, long long points, int fc, int comp, const double* in,
+                      cudaStream_t s);
+
 // streaming multiprocessors of the current device (queried once per device)
 int device_sms();
 

@@ -63,6 +63,7 @@ struct pic_sim {
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     std::string err;
     long long nalloc_tot = 0;    // na_x*na_y*na_z
+    size_t stage_bytes = 0;      // staging memory of the state's conversions (h.scratch)
     long long pcap = 0;          // particle capacity (the buffer sets hold h.cap slots)
 };
 
