@@ -56,7 +56,7 @@ __host__ __device__ constexpr size_t yee2_smem(int es)
 // dynamic shared memory of the 3D field solver for element size es (bytes)
 __host__ __device__ constexpr size_t yee3_smem(int es)
 {
-    return Y3_NS * round128(9ull * Y3_BX * Y3_BY * es) + round128(9ull * Y3_BX * Y3_BY * es) +
+    return Y3_NS * round128(9ull * Y3_BX * Y3_BY * es) + round128(6ull * Y3_BX * Y3_BY * es) +
            round128(6ull * Y3_BX * Y3_BY * es) + round128(12ull * Y3_PX * Y3_PY * es);
 }
 

@@ -18,6 +18,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "beam.cuh"
 #include "sff_common.cuh"
@@ -582,7 +583,13 @@ __global__ void __launch_bounds__(NT, 2) k_yee2r1(const __grid_constant__ SimDev
 //   D(k): B^{n+1} on plane k from Bh(k), N(k), N(k+1); E^{n+1}, B^{n+1} of plane k leave
 //         by one TMA store (double-buffered) and J_{1-p} of plane k is cleared; a column
 //         that ends at x = n_x (y = n_y) also writes that node plane with plain stores,
-// iteration q runs A(q+1) together with D(q-1), then B(q+1): two barriers per plane.
+// iteration q runs A(q+1) together with D(q-1), then B(q+1): two barriers per plane.  A thread
+// keeps its own point's E, Bh and N of the planes on the way in registers; shared memory serves
+// the neighbours' values (21 loads per point and plane, 39 without), and the loop is unrolled over
+// the ring: 0.617 -> 0.589 ms on 512 x 256 x 256.  What bounds it now is the chain of two barriers
+// per plane at 24 warps per SM (issue slots 67 % busy while a block runs, DRAM 2.6 of 6.8 TB/s):
+// leaving out the loads and the clearing of J where no electron is (80 % of this box) changed
+// nothing (0.594 against 0.600 ms).
 // Bh is kept for x in [x0-2, x0+PX], y in [y0-2, y0+PY] and planes from z0-1; N for x in
 // [x0-1, x0+PX], y in [y0-1, y0+PY] and planes from z0: one more point than the outputs need
 // on the low side in x and y, so that every face point's Mur neighbour (one point inwards)
@@ -597,12 +604,11 @@ __device__ __forceinline__ void yee3s_body(const SimDev* __restrict__ sims, cons
     constexpr size_t STAGE = round128(9 * BV * sizeof(R));
     constexpr size_t JOFF = round128(6 * BV * sizeof(R));
     constexpr size_t HOFF = NS * STAGE;
-    constexpr size_t NOFF = HOFF + round128(9 * BV * sizeof(R));
+    constexpr size_t NOFF = HOFF + round128(6 * BV * sizeof(R));
     constexpr size_t OOFF = NOFF + round128(6 * BV * sizeof(R));
     constexpr int AH = PY + 3;                   // Bh range: box x 2 .. PX+4, y 0 .. PY+2
     constexpr int NW = PX + 2, NH = PY + 2;      // N range:  box x 3 .. PX+4, y 1 .. PY+2
     constexpr int NE = 3 * PY + 8;               // Bh points off the core rows (see below)
-    constexpr int NR = 1;                        // Bh points per thread
     static_assert(PX == 32 && NT == 32 * (AH + (NE + 31) / 32), "one warp per row of 32 points, plus the rest");
     static_assert((NS & (NS - 1)) == 0, "a ring of a power-of-two number of stages");
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -615,7 +621,7 @@ __device__ __forceinline__ void yee3s_body(const SimDev* __restrict__ sims, cons
     }
     __syncthreads();
     auto In = [&](int stage) { return reinterpret_cast<R*>(smem_raw + stage * STAGE); };   // [9][BY][BX]
-    R* Hr = reinterpret_cast<R*>(smem_raw + HOFF);     // [3][3][BY][BX]  Bh ring
+    R* Hr = reinterpret_cast<R*>(smem_raw + HOFF);     // [2][3][BY][BX]  Bh ring
     R* Nr = reinterpret_cast<R*>(smem_raw + NOFF);     // [2][3][BY][BX]  N ring
     R* Outb = reinterpret_cast<R*>(smem_raw + OOFF);   // [2][6][PY][PX]
     // Every phase of a plane works on the thread's own point of the Bh range: Bh on all of
@@ -624,8 +630,8 @@ __device__ __forceinline__ void yee3s_body(const SimDev* __restrict__ sims, cons
     // conflicts in any phase); the last warp holds the rest of the range, x = 2 (y >= 1: Bh
     // at (2, 0) feeds nothing), x = 3 and x = PX+4.  Box indices and output slots are fixed
     // for the launch.
-    int pidx[NR], pout[NR];
-    bool pN[NR];
+    int pi, po;
+    bool pN;
     {
         const int w = tid >> 5, lane = tid & 31;
         int lx = 4 + lane, ly = w;
@@ -644,12 +650,11 @@ __device__ __forceinline__ void yee3s_body(const SimDev* __restrict__ sims, cons
                 ly = e - (2 * PY + 5);
             }
         }
-        pidx[0] = has ? lx + BX * ly : -1;
-        pN[0] = has && lx >= 3 && ly >= 1;
-        pout[0] = (has && lx >= 4 && lx < PX + 4 && ly >= 2 && ly < PY + 2) ? (lx - 4) + PX * (ly - 2) : -1;
+        pi = has ? lx + BX * ly : -1;
+        pN = has && lx >= 3 && ly >= 1;
+        po = (has && lx >= 4 && lx < PX + 4 && ly >= 2 && ly < PY + 2) ? (lx - 4) + PX * (ly - 2) : -1;
     }
     uint32_t ph = 0;      // mbarrier phase of each stage
-    int oslot = 0;
     for (;;) {
         if (tid == 0) s_item = atomicAdd(counter, 1);
         __syncthreads();
@@ -681,22 +686,19 @@ __device__ __forceinline__ void yee3s_body(const SimDev* __restrict__ sims, cons
         // column starts there, so this one also writes the node plane x = n_x (y = n_y);
         // and the point's J_{1-p} (cleared for the next step's deposit) on plane -G
         const bool xend = x0 + PX == n0, yend = y0 + PY == n1;
-        unsigned pm[NR];
-        R* jrow[NR];
-#pragma unroll
-        for (int r = 0; r < NR; ++r) {
-            const int gx = x0 - 4 + pidx[r] % BX, gy = y0 - 2 + pidx[r] / BX;
+        unsigned pm;
+        R* jrow;
+        {
+            const int gx = x0 - 4 + pi % BX, gy = y0 - 2 + pi / BX;
             const bool past = (xend && gx == n0 && gy >= y0 && gy <= y0 + PY - (yend ? 0 : 1)) ||
                               (yend && gy == n1 && gx >= x0 && gx <= x0 + PX - (xend ? 0 : 1));
-            pm[r] = (gx == 0 || gx == n0 ? 1u : 0u) | (gy == 0 || gy == n1 ? 2u : 0u) |
-                    (gx >= 0 && gx <= n0 - 1 ? 4u : 0u) | (gx >= 0 && gx <= n0 ? 8u : 0u) |
-                    (gy >= 0 && gy <= n1 - 1 ? 16u : 0u) | (gy >= 0 && gy <= n1 ? 32u : 0u) |
-                    (gx == 0 ? 64u : 0u) | (gy == 0 ? 128u : 0u) | (past ? 256u : 0u);
-            jrow[r] = reinterpret_cast<R*>(S.F) + (long long)comp_j(1 - par) * sc + (long long)(gy + G) * S.sy +
-                      (gx + GX);
+            pm = (gx == 0 || gx == n0 ? 1u : 0u) | (gy == 0 || gy == n1 ? 2u : 0u) |
+                 (gx >= 0 && gx <= n0 - 1 ? 4u : 0u) | (gx >= 0 && gx <= n0 ? 8u : 0u) |
+                 (gy >= 0 && gy <= n1 - 1 ? 16u : 0u) | (gy >= 0 && gy <= n1 ? 32u : 0u) |
+                 (gx == 0 ? 64u : 0u) | (gy == 0 ? 128u : 0u) | (past ? 256u : 0u);
+            jrow = reinterpret_cast<R*>(S.F) + (long long)comp_j(1 - par) * sc + (long long)(gy + G) * S.sy + (gx + GX);
         }
         auto stage_of = [&](int p) { return (p - pa) & (NS - 1); };
-        auto Hs = [&](int p) { return Hr + ((p - pa) % 3) * 3 * BV; };
         auto Ns = [&](int p) { return Nr + ((p - pa) & 1) * 3 * BV; };
         auto issue = [&](int p) {
             const int sgi = stage_of(p);
@@ -768,102 +770,111 @@ __device__ __forceinline__ void yee3s_body(const SimDev* __restrict__ sims, cons
         };
 
 
+        // The thread's own values of the planes on the way stay in registers: E of plane q+1
+        // (e0), Bh of planes q and q-1 (hB, hC), N of planes q and q-1 (nB, nC)
+        R e0[3] = {R(0), R(0), R(0)}, hB[3] = {R(0), R(0), R(0)}, hC[3] = {R(0), R(0), R(0)};
+        R nB[3] = {R(0), R(0), R(0)}, nC[3] = {R(0), R(0), R(0)};
         bool failed = false;
-        for (int q = z0 - 2; q <= z1; ++q) {
+        // One iteration per plane: q = z0 - 2 + k, unrolled over the ring (K = k mod NS), so that
+        // every stage and slot is a constant and every shared-memory access an immediate offset.
+        // False: the loop is over or a wait gave up.
+        auto plane = [&](auto KC, int k) -> bool {
+            constexpr int K = decltype(KC)::value;
+            constexpr int S1 = K, S2 = (K + 1) % NS;      // stages of planes q+1, q+2
+            constexpr int C = K & 1;                      // slot of planes q+1, q-1 (Bh, N, output)
+            const int q = z0 - 2 + k;
+            if (q > z1) return false;
             // Plane q was last read in the previous iteration unless this one's z-face passes
             // read it (B(n_z) reads E(n_z - 1), the plane-0 faces E(0)): otherwise its stage
             // takes plane q+NS as soon as this iteration's first barrier has passed
             const bool early = q + 1 != n2 && q + 1 != 1;
             bool ok = true;
-            while (pw < min(q + 2, plast)) {
-                ++pw;
-                const int sgi = stage_of(pw);
-                ok = ok && mbar_wait_bounded(&bars[sgi], (ph >> sgi) & 1u);
-                ph ^= 1u << sgi;
+            if (k == 0) {
+                ok = mbar_wait_bounded(&bars[S1], (ph >> S1) & 1u);
+                ph ^= 1u << S1;
+                pw = pa;
             }
-            // S1: A(q+1) and D(q-1) on the thread's points
+            if (q + 2 <= plast) {
+                ok = ok && mbar_wait_bounded(&bars[S2], (ph >> S2) & 1u);
+                ph ^= 1u << S2;
+                pw = q + 2;
+            }
+            // S1: D(q-1) and A(q+1) on the thread's point
             const bool doA = q + 1 <= z1, doD = q - 1 >= z0;
-            if (doA || doD) {
-                const int m = q - 1;
-                const R* I0 = In(stage_of(q + 1));
-                const R* I1 = In(stage_of(q + 2));
-                R* Ha = doA ? Hs(q + 1) : Hr;
-                const R* H0 = doD ? Hs(m) : Hr;
-                const R* N0 = Ns(m + 2);
-                const R* N1 = Ns(m + 1);
-                R* Out = Outb + oslot * 6 * TV;
-                // every output point of the plane has all six components
-                const bool zint = col_int && m >= 1 && m <= n2 - 1;
-                const bool zs = m >= 0 && m <= n2 - 1, zn = m >= 0 && m <= n2;
-                const long long zoff = (long long)(m + G) * sz;
-#pragma unroll
-                for (int r = 0; r < NR; ++r) {
-                    const int i = pidx[r];
-                    if (i < 0) continue;
-                    if (doD && (pout[r] >= 0 || (pm[r] & 256u))) {
-                        const R dNz_dy = N0[2 * BV + i + BX] - N0[2 * BV + i];
-                        const R dNx_dy = N0[i + BX] - N0[i];
-                        const R dNy_dz = N1[BV + i] - N0[BV + i];
-                        const R dNx_dz = N1[i] - N0[i];
-                        const R dNz_dx = N0[2 * BV + i + 1] - N0[2 * BV + i];
-                        const R dNy_dx = N0[BV + i + 1] - N0[BV + i];
-                        R v[6] = {N0[i], N0[BV + i], N0[2 * BV + i], H0[i] - hc * (dNz_dy - dNy_dz),
-                                  H0[BV + i] - hc * (dNx_dz - dNz_dx), H0[2 * BV + i] - hc * (dNy_dx - dNx_dy)};
-                        if (!zint) {
-                            const unsigned b = pm[r];
-                            const bool xs = b & 4u, xn = b & 8u, ys = b & 16u, yn = b & 32u;
-                            if (!(xs && yn && zn)) v[0] = R(0);
-                            if (!(xn && ys && zn)) v[1] = R(0);
-                            if (!(xn && yn && zs)) v[2] = R(0);
-                            if (!(xn && ys && zs)) v[3] = R(0);
-                            if (!(xs && yn && zs)) v[4] = R(0);
-                            if (!(xs && ys && zn)) v[5] = R(0);
-                        }
-                        const int u = pout[r];
-                        R* jp = jrow[r] + zoff;
-                        if (u >= 0) {
-#pragma unroll
-                            for (int c = 0; c < 6; ++c) Out[c * TV + u] = v[c];
-                        } else {
-                            // past the tile (node plane x = n_x / y = n_y): plain stores
-                            R* ep = jp + (long long)(comp_eb(1 - par) - comp_j(1 - par)) * sc;
-#pragma unroll
-                            for (int c = 0; c < 6; ++c) ep[c * sc] = v[c];
-                        }
-                        // clear J_{1-p} on plane m (the next step deposits into it)
-                        jp[0] = R(0);
-                        jp[sc] = R(0);
-                        jp[2 * sc] = R(0);
-                    }
-                    if (doA) {
-                        const R dEz_dy = I0[2 * BV + i + BX] - I0[2 * BV + i];
-                        const R dEx_dy = I0[i + BX] - I0[i];
-                        const R dEy_dz = I1[BV + i] - I0[BV + i];
-                        const R dEx_dz = I1[i] - I0[i];
-                        const R dEz_dx = I0[2 * BV + i + 1] - I0[2 * BV + i];
-                        const R dEy_dx = I0[BV + i + 1] - I0[BV + i];
-                        Ha[i] = I0[3 * BV + i] - hc * (dEz_dy - dEy_dz);
-                        Ha[BV + i] = I0[4 * BV + i] - hc * (dEx_dz - dEz_dx);
-                        Ha[2 * BV + i] = I0[5 * BV + i] - hc * (dEy_dx - dEx_dy);
-                    }
+            if (doD && (po >= 0 || (pm & 256u))) {
+                const int m = q - 1, i = pi;
+                const R* N0 = Nr + C * 3 * BV;  // plane m (a ring of two)
+                const R dNz_dy = N0[2 * BV + i + BX] - nC[2];
+                const R dNx_dy = N0[i + BX] - nC[0];
+                const R dNz_dx = N0[2 * BV + i + 1] - nC[2];
+                const R dNy_dx = N0[BV + i + 1] - nC[1];
+                const R dNy_dz = nB[1] - nC[1];
+                const R dNx_dz = nB[0] - nC[0];
+                R v[6] = {nC[0], nC[1], nC[2], hC[0] - hc * (dNz_dy - dNy_dz), hC[1] - hc * (dNx_dz - dNz_dx),
+                          hC[2] - hc * (dNy_dx - dNx_dy)};
+                if (!(col_int && m >= 1 && m <= n2 - 1)) {
+                    const bool zs = m >= 0 && m <= n2 - 1, zn = m >= 0 && m <= n2;
+                    const bool xs = pm & 4u, xn = pm & 8u, ys = pm & 16u, yn = pm & 32u;
+                    if (!(xs && yn && zn)) v[0] = R(0);
+                    if (!(xn && ys && zn)) v[1] = R(0);
+                    if (!(xn && yn && zs)) v[2] = R(0);
+                    if (!(xn && ys && zs)) v[3] = R(0);
+                    if (!(xs && yn && zs)) v[4] = R(0);
+                    if (!(xs && ys && zn)) v[5] = R(0);
                 }
+                R* Out = Outb + C * 6 * TV;
+                R* jp = jrow + (long long)(m + G) * sz;
+                if (po >= 0) {
+#pragma unroll
+                    for (int c = 0; c < 6; ++c) Out[c * TV + po] = v[c];
+                } else {
+                    // past the tile (node plane x = n_x / y = n_y): plain stores
+                    R* ep = jp + (long long)(comp_eb(1 - par) - comp_j(1 - par)) * sc;
+#pragma unroll
+                    for (int c = 0; c < 6; ++c) ep[c * sc] = v[c];
+                }
+                // clear J_{1-p} on plane m (the next step deposits into it)
+                jp[0] = R(0);
+                jp[sc] = R(0);
+                jp[2 * sc] = R(0);
+            }
+            R hA[3] = {R(0), R(0), R(0)}, e1[3] = {R(0), R(0), R(0)}, nA[3] = {R(0), R(0), R(0)};
+            if (doA && pi >= 0) {
+                const int i = pi;
+                const R* I0 = In(S1);
+                const R* I1 = In(S2);
+                R* Ha = Hr + C * 3 * BV;
+                if (k == 0) {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) e0[c] = I0[c * BV + i];
+                }
+#pragma unroll
+                for (int c = 0; c < 3; ++c) e1[c] = I1[c * BV + i];
+                const R dEz_dy = I0[2 * BV + i + BX] - e0[2];
+                const R dEx_dy = I0[i + BX] - e0[0];
+                const R dEz_dx = I0[2 * BV + i + 1] - e0[2];
+                const R dEy_dx = I0[BV + i + 1] - e0[1];
+                const R dEy_dz = e1[1] - e0[1];
+                const R dEx_dz = e1[0] - e0[0];
+                hA[0] = I0[3 * BV + i] - hc * (dEz_dy - dEy_dz);
+                hA[1] = I0[4 * BV + i] - hc * (dEx_dz - dEz_dx);
+                hA[2] = I0[5 * BV + i] - hc * (dEy_dx - dEx_dy);
+#pragma unroll
+                for (int c = 0; c < 3; ++c) Ha[c * BV + i] = hA[c];
             }
             if (doD) fence_proxy_async_smem();
             if (__syncthreads_or(!ok)) {
                 failed = true;
-                break;
+                return false;
             }
             if (early && q >= pa && q + NS <= plast) {
                 if (tid == 0) issue(q + NS);
                 pissued = q + NS;
             }
-            if (doD) {
-                if (tid == 0) {
-                    const int oc[3] = {x0 + GX, y0 + G, q - 1 + G};
-                    tma_store_box<3>(&S.tm_yout, oc, comp_eb(1 - par), Outb + oslot * 6 * TV);
-                    bulk_commit();
-                }
-                oslot ^= 1;
+            if (doD && tid == 0) {
+                const int oc[3] = {x0 + GX, y0 + G, q - 1 + G};
+                tma_store_box<3>(&S.tm_yout, oc, comp_eb(1 - par), Outb + C * 6 * TV);
+                bulk_commit();
             }
             // S2: B(q+1) on the thread's points of the N range, with the Mur condition on the
             // x and y faces; on the z faces the passes of mur_plane follow
@@ -871,70 +882,76 @@ __device__ __forceinline__ void yee3s_body(const SimDev* __restrict__ sims, cons
             if (b >= z0 && b <= z1) {
                 const bool fz = b == 0 || b == n2;
                 const bool faces = !col_int || fz;
-                const R* I0 = In(stage_of(b));
+                const R* I0 = In(S1);
                 const R* J0 = I0 + JOFF / sizeof(R);
-                const R* Hc = Hs(b);
-                const R* Hp = Hs(b + 2);      // plane b-1 (a ring of three)
-                R* Nc = Ns(b);
-                // E^{n+1} component c at box point j (backward differences of Bh)
-                auto enew = [&](int c, int j) -> R {
-                    if (c == 0) {
-                        const R dBz_dy = Hc[2 * BV + j] - Hc[2 * BV + j - BX];
-                        const R dBy_dz = Hc[BV + j] - Hp[BV + j];
-                        return I0[j] + cdt * (dBz_dy - dBy_dz) - dt * J0[j];
-                    } else if (c == 1) {
-                        const R dBx_dz = Hc[j] - Hp[j];
-                        const R dBz_dx = Hc[2 * BV + j] - Hc[2 * BV + j - 1];
-                        return I0[BV + j] + cdt * (dBx_dz - dBz_dx) - dt * J0[BV + j];
-                    }
-                    const R dBy_dx = Hc[BV + j] - Hc[BV + j - 1];
-                    const R dBx_dy = Hc[j] - Hc[j - BX];
-                    return I0[2 * BV + j] + cdt * (dBy_dx - dBx_dy) - dt * J0[2 * BV + j];
-                };
-                // first-order Mur at face point j of component c from the inward neighbour nb
-                // (E^n from the stage, E^{n+1} of the neighbour given)
-                auto mur = [&](int c, int j, int nb, R en_nb) -> R {
-                    return I0[c * BV + nb] + km * (en_nb - I0[c * BV + j]);
-                };
-#pragma unroll
-                for (int r = 0; r < NR; ++r) {
-                    if (!pN[r]) continue;
-                    const int i = pidx[r];
-                    const R ex = enew(0, i), ey = enew(1, i), ez = enew(2, i);
-                    const unsigned f = pm[r];
+                const R* Hb = Hr + C * 3 * BV;
+                const R* Hp = Hr + (1 - C) * 3 * BV;      // plane b-1
+                R* Nc = Nr + C * 3 * BV;
+                auto less_j = [&](R e, int k) -> R { return e - dt * J0[k]; };
+                if (pN) {
+                    const int i = pi;
+                    // E^{n+1} at the thread's point (backward differences of Bh; plane b-1: hB)
+                    R n[3] = {less_j(e0[0] + cdt * ((hA[2] - Hb[2 * BV + i - BX]) - (hA[1] - hB[1])), i),
+                              less_j(e0[1] + cdt * ((hA[0] - hB[0]) - (hA[2] - Hb[2 * BV + i - 1])), BV + i),
+                              less_j(e0[2] + cdt * ((hA[1] - Hb[BV + i - 1]) - (hA[0] - Hb[i - BX])), 2 * BV + i)};
+                    const unsigned f = pm;
                     const bool fx = f & 1u, fy = f & 2u;
-                    if (!faces || (!fx && !fy && !fz)) {
-                        Nc[i] = ex;
-                        Nc[BV + i] = ey;
-                        Nc[2 * BV + i] = ez;
-                    } else if (fz) {
-                        // z faces: every face point is left to mur_plane
-                        if (!(fy || fz)) Nc[i] = ex;
-                        if (!(fx || fz)) Nc[BV + i] = ey;
-                        if (!(fx || fy)) Nc[2 * BV + i] = ez;
-                    } else {
-                        // x / y faces (points on fewer faces first, along the lowest face axis:
-                        // Ez on an x-y edge takes its x neighbour's value on the y face)
-                        const int sx = (f & 64u) ? 1 : -1, sy = (f & 128u) ? BX : -BX;
-                        Nc[i] = fy ? mur(0, i, i + sy, enew(0, i + sy)) : ex;
-                        Nc[BV + i] = fx ? mur(1, i, i + sx, enew(1, i + sx)) : ey;
-                        R vz = ez;
-                        if (fx && fy) {
-                            const int nb = i + sx;
-                            vz = mur(2, i, nb, mur(2, nb, nb + sy, enew(2, nb + sy)));
-                        } else if (fx) {
-                            vz = mur(2, i, i + sx, enew(2, i + sx));
-                        } else if (fy) {
-                            vz = mur(2, i, i + sy, enew(2, i + sy));
+                    if (faces && (fx || fy || fz)) {
+                        // tangential E on a face: first-order Mur from the inward neighbour's E^{n+1},
+                        // evaluated here on the x and y faces (E^n from the stage)
+                        auto mur = [&](int c, int j, int nb, R en_nb) -> R {
+                            return I0[c * BV + nb] + km * (en_nb - I0[c * BV + j]);
+                        };
+                        auto enz = [&](int j) -> R {
+                            return less_j(I0[2 * BV + j] + cdt * ((Hb[BV + j] - Hb[BV + j - 1]) - (Hb[j] - Hb[j - BX])),
+                                          2 * BV + j);
+                        };
+                        auto enx = [&](int j) -> R {
+                            return less_j(I0[j] + cdt * ((Hb[2 * BV + j] - Hb[2 * BV + j - BX]) - (Hb[BV + j] - Hp[BV + j])), j);
+                        };
+                        auto eny = [&](int j) -> R {
+                            return less_j(I0[BV + j] + cdt * ((Hb[j] - Hp[j]) - (Hb[2 * BV + j] - Hb[2 * BV + j - 1])), BV + j);
+                        };
+                        if (fz) {
+                            // z faces: every face point is left to mur_plane
+                            if (!fx && !fy) Nc[2 * BV + i] = n[2];
+                        } else {
+                            // points on fewer faces first, along the lowest face axis: Ez on an x-y
+                            // edge takes its x neighbour's value on the y face
+                            const int sx = (f & 64u) ? 1 : -1, sy = (f & 128u) ? BX : -BX;
+                            if (fy) n[0] = mur(0, i, i + sy, enx(i + sy));
+                            if (fx) n[1] = mur(1, i, i + sx, eny(i + sx));
+                            if (fx && fy) {
+                                const int nb = i + sx;
+                                n[2] = mur(2, i, nb, mur(2, nb, nb + sy, enz(nb + sy)));
+                            } else if (fx) {
+                                n[2] = mur(2, i, i + sx, enz(i + sx));
+                            } else {
+                                n[2] = mur(2, i, i + sy, enz(i + sy));
+                            }
                         }
-                        Nc[2 * BV + i] = vz;
                     }
+                    if (!fz) {
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) Nc[c * BV + i] = n[c];
+                    }
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) nA[c] = n[c];
                 }
                 // the store of two planes back has read its buffer (reused by the next D)
                 if (tid == 0) bulk_wait_read1();
                 __syncthreads();
                 if (fz && b != 0) mur_plane(b);
                 if (b == 1 && z0 <= 1) mur_plane(0);
+                // the z-face passes wrote N of their plane in shared memory
+                if (pN && fz && b != 0) {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) nA[c] = Nc[c * BV + pi];
+                }
+                if (pN && b == 1 && z0 <= 1) {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) nB[c] = Ns(0)[c * BV + pi];
+                }
             } else {
                 if (tid == 0) bulk_wait_read1();
                 __syncthreads();
@@ -944,6 +961,22 @@ __device__ __forceinline__ void yee3s_body(const SimDev* __restrict__ sims, cons
                 if (tid == 0) issue(q + NS);
                 pissued = q + NS;
             }
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                e0[c] = e1[c];
+                hC[c] = hB[c];
+                hB[c] = hA[c];
+                nC[c] = nB[c];
+                nB[c] = nA[c];
+            }
+            return true;
+        };
+        static_assert(NS == 4, "the unrolled loop below");
+        for (int k = 0;; k += NS) {
+            if (!plane(std::integral_constant<int, 0>{}, k)) break;
+            if (!plane(std::integral_constant<int, 1>{}, k + 1)) break;
+            if (!plane(std::integral_constant<int, 2>{}, k + 2)) break;
+            if (!plane(std::integral_constant<int, 3>{}, k + 3)) break;
         }
         if (failed) {
             if (tid == 0) {
