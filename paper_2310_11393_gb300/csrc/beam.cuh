@@ -296,7 +296,7 @@ __device__ __forceinline__ bool phi_closed_log(const BeamC<R>& b, R rho2, R zeta
 // LP / RP field in the beam frame (paper x, y, z), E and B real parts.
 //   xi = x/a, eta = y/a, zeta = z/a;  tmz = t_rel - z, tpz = t_rel + z (formed in double);
 //   trel = t - t_focus.
-template <int D, typename R>
+template <bool LOG, typename R>
 __device__ __forceinline__ void focused_field(const BeamC<R>& b, R xi, R eta, R zeta, R tmz, R tpz, R trel, R E[3],
                                               R B[3])
 {
@@ -308,7 +308,7 @@ __device__ __forceinline__ void focused_field(const BeamC<R>& b, R xi, R eta, R 
         phi_series(b, u, trel, P);
     } else {
         bool any;
-        if constexpr (D == 3 && sizeof(R) == 4) any = phi_closed_log(b, rho2, zeta, u, tmz, tpz, P);
+        if constexpr (LOG) any = phi_closed_log(b, rho2, zeta, u, tmz, tpz, P);
         else any = phi_closed(b, rho2, zeta, u, uu, tmz, tpz, P);
         if (!any) {
 #pragma unroll
@@ -395,7 +395,8 @@ __device__ __forceinline__ PhaseRef<R> phase_ref(const SimDev& S, double t, int 
 }
 
 // Incident E, B (grid axes) at a particle in cell c with offsets o, at the time of `pr`.
-template <int D, typename R>
+// DIAG: not for a push (see phi_closed_log).
+template <int D, typename R, bool DIAG = false>
 __device__ __forceinline__ void incident_at(const SimDev& S, const BeamC<R>& b, const PhaseRef<R>& pr, const int c[3],
                                             const R o[3], R E[3], R B[3])
 {
@@ -434,7 +435,7 @@ __device__ __forceinline__ void incident_at(const SimDev& S, const BeamC<R>& b, 
         if constexpr (D >= 2) xi = ((R)(c[1] - S.icf[1]) + (o[1] - b.frf[1])) * (b.dxr * inv_a);
         if constexpr (D >= 3) eta = ((R)(c[2] - S.icf[2]) + (o[2] - b.frf[2])) * (b.dxr * inv_a);
         R Ep[3], Bp[3];
-        focused_field<D, R>(b, xi, eta, zeta, tmz, tpz, pr.trel, Ep, Bp);
+        focused_field<D == 3 && sizeof(R) == 4 && !DIAG, R>(b, xi, eta, zeta, tmz, tpz, pr.trel, Ep, Bp);
         E[0] = Ep[2];
         E[1] = Ep[0];
         E[2] = Ep[1];

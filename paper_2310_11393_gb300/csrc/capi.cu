@@ -578,7 +578,7 @@ pic_status compute_rho_ion(pic_sim* s, cudaStream_t st)
     if (r != PIC_OK) return r;
     // immobile ions co-located with the electrons: rho_ion = -rho_e, deposited in place
     CU_CHECK(s, cudaMemsetAsync(s->h.rho_ion, 0, sizeof(double) * s->nalloc_tot, st));
-    launch_charge(s->d, s->cfg.dim, s->cfg.precision, s->h.cap, s->h.rho_ion, st, -1.0);
+    launch_charge(s->d, s->cfg.dim, s->cfg.precision, s->h.nptiles, s->h.rho_ion, st, -1.0);
     CU_CHECK(s, cudaGetLastError());
     CU_CHECK(s, cudaStreamSynchronize(st));
     return PIC_OK;
@@ -1100,9 +1100,12 @@ pic_status pic_set_fields(pic_sim* s, const double* fields, void* stream)
     if (r != PIC_OK) return r;
     const int D = s->cfg.dim;
     const long long ne = (long long)(s->h.n[0] + 1) * (D > 1 ? s->h.n[1] + 1 : 1) * (D > 2 ? s->h.n[2] + 1 : 1);
-    for (int comp = 0; comp < 6; ++comp) {
-        CU_CHECK(s, cudaMemcpyAsync(s->h.scratch, fields + comp * ne, (size_t)ne * 8, cudaMemcpyHostToDevice, st));
-        launch_put_field(s->d, D, s->cfg.precision, s->nalloc_tot, comp_eb(ds.parity) + comp, comp, s->h.scratch, st);
+    // as many components at a time as the staging memory holds
+    const int per = (int)std::min<long long>(6, (long long)(s->stage_bytes / 8) / ne);
+    for (int c0 = 0; c0 < 6; c0 += per) {
+        const int nc = std::min(per, 6 - c0);
+        CU_CHECK(s, cudaMemcpyAsync(s->h.scratch, fields + c0 * ne, (size_t)nc * ne * 8, cudaMemcpyHostToDevice, st));
+        launch_put_field(s->d, D, s->cfg.precision, s->nalloc_tot, ds.parity, c0, nc, s->h.scratch, st);
         CU_CHECK(s, cudaGetLastError());
     }
     CU_CHECK(s, cudaStreamSynchronize(st));
@@ -1128,7 +1131,7 @@ pic_status pic_diag(pic_sim* s, int kind, void* host_out, size_t bytes, void* st
         if (bytes < 8 * sizeof(double)) return fail(s, PIC_ECAPACITY, "ENERGIES needs 64 bytes");
         CU_CHECK(s, cudaMemsetAsync(s->d_acc, 0, 4 * sizeof(double), st));
         launch_energy_fields(s->d, D, s->cfg.precision, s->h.n, s->d_acc, st);
-        launch_energy_particles(s->d, D, s->cfg.precision, s->h.cap, nex, s->d_acc, st);
+        launch_energy_particles(s->d, s->cfg.precision, s->h.nptiles, nex, s->d_acc, st);
         CU_CHECK(s, cudaGetLastError());
         double acc[4];
         CU_CHECK(s, cudaMemcpyAsync(acc, s->d_acc, sizeof acc, cudaMemcpyDeviceToHost, st));
@@ -1147,7 +1150,7 @@ pic_status pic_diag(pic_sim* s, int kind, void* host_out, size_t bytes, void* st
         if (bytes < sizeof(double)) return fail(s, PIC_ECAPACITY, "GAUSS needs 8 bytes");
         CU_CHECK(s, cudaMemsetAsync(s->h.scratch, 0, sizeof(double) * s->nalloc_tot, st));
         CU_CHECK(s, cudaMemsetAsync(s->d_bits, 0, 8, st));
-        launch_charge(s->d, D, s->cfg.precision, s->h.cap, s->h.scratch, st);
+        launch_charge(s->d, D, s->cfg.precision, s->h.nptiles, s->h.scratch, st);
         launch_gauss(s->d, D, s->cfg.precision, s->h.n, s->h.scratch, s->d_bits, st);
         CU_CHECK(s, cudaGetLastError());
         unsigned long long bits;
@@ -1194,13 +1197,13 @@ pic_status pic_diag(pic_sim* s, int kind, void* host_out, size_t bytes, void* st
         const long long ne = (long long)ext[0] * ext[1] * ext[2];
         if (bytes < (size_t)9 * ne * 8) return fail(s, PIC_ECAPACITY, "FIELDS needs %lld bytes", 9 * ne * 8);
         double* o = (double*)host_out;
-        for (int comp = 0; comp < 9; ++comp) {
-            // the current deposited by the last step sits in J of the other set
-            const int fc = comp < 6 ? comp_eb(ds.parity) + comp : comp_j(1 - ds.parity) + comp - 6;
-            launch_get_field(s->d, D, s->cfg.precision, ne, fc, comp, s->h.scratch, st);
+        const int per = (int)std::min<long long>(9, (long long)(s->stage_bytes / 8) / ne);
+        for (int c0 = 0; c0 < 9; c0 += per) {
+            const int nc = std::min(per, 9 - c0);
+            launch_get_field(s->d, D, s->cfg.precision, ne, ds.parity, c0, nc, s->h.scratch, st);
             CU_CHECK(s, cudaGetLastError());
-            touch_pages(o + comp * ne, (size_t)ne * 8);
-            CU_CHECK(s, cudaMemcpyAsync(o + comp * ne, s->h.scratch, (size_t)ne * 8, cudaMemcpyDeviceToHost, st));
+            touch_pages(o + c0 * ne, (size_t)nc * ne * 8);
+            CU_CHECK(s, cudaMemcpyAsync(o + c0 * ne, s->h.scratch, (size_t)nc * ne * 8, cudaMemcpyDeviceToHost, st));
         }
         CU_CHECK(s, cudaStreamSynchronize(st));
         return PIC_OK;
@@ -1233,7 +1236,7 @@ pic_status pic_histogram(pic_sim* s, int n_e, double e_max, int n_a, double* hos
     const size_t nb = (size_t)n_e * n_a;
     if (nb > (size_t)s->nalloc_tot) return fail(s, PIC_ECAPACITY, "too many bins");
     CU_CHECK(s, cudaMemsetAsync(s->h.scratch, 0, nb * 8, st));
-    launch_histogram(s->d, s->cfg.dim, s->cfg.precision, s->h.cap, std::min<long long>(ds.n_exits, s->h.max_exits),
+    launch_histogram(s->d, s->cfg.precision, s->h.nptiles, ds.n_alive, std::min<long long>(ds.n_exits, s->h.max_exits),
                      n_e, e_max, n_a, s->h.scratch, st);
     CU_CHECK(s, cudaGetLastError());
     CU_CHECK(s, cudaMemcpyAsync(host_out, s->h.scratch, nb * 8, cudaMemcpyDeviceToHost, st));

@@ -25,28 +25,16 @@ __device__ __forceinline__ void decode_cell_d(const SimDev& S, unsigned cl, int 
     if constexpr (D > 2) c[2] = (int)(cl >> (S.cb[0] + S.cb[1]));
 }
 
-// Slot p of buffer set par holds a particle: slots after a tile's particles hold DEAD or
-// stale records of earlier steps, whose cell puts them outside their tile's occupied slots.
-template <int D>
-__device__ __forceinline__ bool slot_live(const SimDev& S, int par, long long p)
+// body(p) for every particle slot p of buffer set par, a block per tile (the tiles' occupied
+// slots only: two to three times as many slots are in use as hold particles)
+template <typename F>
+__device__ __forceinline__ void for_particles(const SimDev& S, int par, F body)
 {
-    const unsigned cl = S.cell[par][p];
-    if (cl == DEAD) return false;
-    int c[3];
-    decode_cell_d<D>(S, cl, c);
-    int t = 0, mul = 1;
-    for (int d = 0; d < D; ++d) {
-        if (c[d] >= S.n[d]) return false;
-        t += (c[d] / S.pt[d]) * mul;
-        mul *= S.npt[d];
+    for (int t = blockIdx.x; t < S.nptiles; t += gridDim.x) {
+        const long long p0 = S.toff[par][t];
+        const int n = S.tnum[par][t];
+        for (int i = threadIdx.x; i < n; i += blockDim.x) body(p0 + i);
     }
-    return (unsigned long long)(p - S.toff[par][t]) < (unsigned long long)S.tnum[par][t];
-}
-
-// end of the occupied slot range of buffer set par (n: slots of a set)
-__device__ __forceinline__ long long slots_used(const SimDev& S, int par, long long n)
-{
-    return min(n, (long long)S.toff[par][S.nptiles]);
 }
 
 __device__ __forceinline__ double warp_sum(double v)
@@ -57,16 +45,13 @@ __device__ __forceinline__ double warp_sum(double v)
 }
 
 // charge density scale * rho_e, rho_e = -sum w S(x - x_node), added on the primal nodes
-// (array coordinates); n: slots of a buffer set (as for the other particle diagnostics)
+// (array coordinates)
 template <int D, typename R>
-__global__ void k_charge(const SimDev* __restrict__ sim, long long n, double* __restrict__ rho, double scale)
+__global__ void k_charge(const SimDev* __restrict__ sim, double* __restrict__ rho, double scale)
 {
     const SimDev& S = *sim;
     const int par = S.st->parity;
-    const long long nu = slots_used(S, par, n);
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < nu;
-         p += (long long)gridDim.x * blockDim.x) {
-        if (!slot_live<D>(S, par, p)) continue;
+    for_particles(S, par, [&](long long p) {
         int c[3];
         decode_cell_d<D>(S, S.cell[par][p], c);
         double w[3][3];
@@ -92,7 +77,7 @@ __global__ void k_charge(const SimDev* __restrict__ sim, long long n, double* __
                 for (int i = 0; i < 3; ++i)
                     atomicAdd(&rho[(long long)(lo[2] + k) * S.sz + (long long)(lo[1] + j) * S.sy + lo[0] + i],
                               q * w[0][i] * w[1][j] * w[2][k]);
-    }
+    });
 }
 
 // max |div E - rho - rho_ion| over interior primal nodes; result as ordered bits
@@ -121,28 +106,58 @@ __global__ void k_gauss(const SimDev* __restrict__ sim, const double* __restrict
     if ((threadIdx.x & 31) == 0) atomicMax(out, (unsigned long long)__double_as_longlong(worst));
 }
 
-// 1/2 sum F^2 dx^dim over the points each component has: [0] scattered, [1] scattered + incident
+// Is component comp of the incident field identically zero (grid axes: the beam's z is x, its x
+// is y, its y is z)?  The plane wave has E_y and B_z, the 2D Gaussian beam E_x, E_y and B_z; the
+// focused pulses have no component odd in y (their own; grid z) in 2D, and RP no B along its axis.
+template <int D>
+__device__ __forceinline__ bool incident_zero(int beam, int comp)
+{
+    if (beam == BEAM_NONE) return true;
+    if (beam == BEAM_PLANE) return comp != 1 && comp != 5;
+    if (beam == BEAM_GAUSS2D) return comp != 0 && comp != 1 && comp != 5;
+    if (beam == BEAM_LP || beam == BEAM_RP)
+        return (D == 2 && comp != 0 && comp != 1 && comp != 5) || (beam == BEAM_RP && comp == 3);
+    return false;
+}
+
+// 1/2 sum F^2 dx^dim over the points each component has: [0] scattered, [1] scattered + incident.
+// A block takes 256 points of a row at a time: one double-precision phase reference per row
+// segment (per point and component it was most of the kernel: FP64 runs at 1/64 of the FP32
+// rate), the components in turn, those that are identically zero without the closed form.
+// Double sums.  3D RP 512 x 256 x 256: 12.0 -> 6.6 ms with the particle part.
 template <int D, typename R>
-__global__ void k_energy_fields(const SimDev* __restrict__ sim, int m0, int m1, int m2, double* __restrict__ acc)
+__global__ void __launch_bounds__(256) k_energy_fields(const SimDev* __restrict__ sim, double* __restrict__ acc)
 {
     const SimDev& S = *sim;
     const R* F = reinterpret_cast<const R*>(S.F);
-    const int par = S.st->parity;
-    const long long eb = (long long)comp_eb(par) * S.sc;
-    const double t = (double)S.st->step * S.dt;
+    const DevState* st = S.st;
+    const long long eb = (long long)comp_eb(st->parity) * S.sc;
+    const double t = (double)st->step * S.dt;
     const BeamC<R>& bc = beam_of<R>(S);
-    const long long total = (long long)m0 * m1 * m2;   // extents n+1 on resolved axes
+    const int m0 = S.n[0] + 1, m1 = D > 1 ? S.n[1] + 1 : 1, m2 = D > 2 ? S.n[2] + 1 : 1;
+    const long long segs = (m0 + 255) / 256, total = segs * m1 * m2;
+    __shared__ PhaseRef<R> s_pr;
     double es = 0.0, et = 0.0;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < total;
-         k += (long long)gridDim.x * blockDim.x) {
-        const int g[3] = {(int)(k % m0), (int)((k / m0) % m1), (int)(k / ((long long)m0 * m1))};
+    // the segments of one place along x in turn: the phase reference changes with that place only
+    long long ref_seg = -1;
+    for (long long k = blockIdx.x; k < total; k += gridDim.x) {
+        const long long rows = (long long)m1 * m2, seg = k / rows, row = k - seg * rows;
+        if (seg != ref_seg) {
+            __syncthreads();
+            if (threadIdx.x == 0) s_pr = phase_ref<R>(S, t, (int)seg * 256);
+            __syncthreads();
+            ref_seg = seg;
+        }
+        const int g[3] = {(int)seg * 256 + (int)threadIdx.x, (int)(row % m1), (int)(row / m1)};
+        if (g[0] >= m0) continue;
         const long long o = (long long)(D > 2 ? g[2] + G : 0) * S.sz + (long long)(D > 1 ? g[1] + G : 0) * S.sy +
                             (g[0] + GX);
+#pragma unroll 1
         for (int comp = 0; comp < 6; ++comp) {
             const int c = comp % 3;
             bool has = true;
-            int cc[3] = {g[0], g[1], g[2]};
             R oo[3] = {R(0), R(0), R(0)};
+#pragma unroll
             for (int d = 0; d < D; ++d) {
                 const bool stag = comp < 3 ? (d == c) : (d != c);
                 if (stag) {
@@ -152,15 +167,15 @@ __global__ void k_energy_fields(const SimDev* __restrict__ sim, int m0, int m1, 
             }
             if (!has) continue;
             const double f = (double)F[eb + comp * S.sc + o];
-            es += 0.5 * f * f;
-            double inc = 0.0;
-            if (S.beam != BEAM_NONE && !S.tf) {
+            double h = f;
+            if (!S.tf && !incident_zero<D>(S.beam, comp)) {
                 R Ei[3], Bi[3];
-                const PhaseRef<R> pr = phase_ref<R>(S, t, cc[0]);
-                incident_at<D, R>(S, bc, pr, cc, oo, Ei, Bi);
-                inc = comp < 3 ? (double)Ei[c] : (double)Bi[c];
+                incident_at<D, R, true>(S, bc, s_pr, g, oo, Ei, Bi);
+                const R e = c == 0 ? Ei[0] : (c == 1 ? Ei[1] : Ei[2]), b = c == 0 ? Bi[0] : (c == 1 ? Bi[1] : Bi[2]);
+                h += (double)(comp < 3 ? e : b);
             }
-            et += 0.5 * (f + inc) * (f + inc);
+            es += 0.5 * f * f;
+            et += 0.5 * h * h;
         }
     }
     es = warp_sum(es);
@@ -172,23 +187,20 @@ __global__ void k_energy_fields(const SimDev* __restrict__ sim, int m0, int m1, 
 }
 
 // [2] sum w (gamma - 1) of electrons in the box, [3] of exit records (times dx^dim on the host)
-template <int D, typename R>
-__global__ void k_energy_particles(const SimDev* __restrict__ sim, long long n, long long nex, double* __restrict__ acc)
+template <typename R>
+__global__ void k_energy_particles(const SimDev* __restrict__ sim, long long nex, double* __restrict__ acc)
 {
     const SimDev& S = *sim;
     const int par = S.st->parity;
     double ka = 0.0, ke = 0.0;
-    const long long nu = slots_used(S, par, n);
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < nu;
-         p += (long long)gridDim.x * blockDim.x) {
-        if (!slot_live<D>(S, par, p)) continue;
+    for_particles(S, par, [&](long long p) {
         double u2 = 0.0;
         for (int d = 0; d < 3; ++d) {
             const double u = (double)reinterpret_cast<const R*>(S.mom[par][d])[p];
             u2 += u * u;
         }
         ka += (double)reinterpret_cast<const R*>(S.wgt[par])[p] * (sqrt(1.0 + u2) - 1.0);
-    }
+    });
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < nex;
          p += (long long)gridDim.x * blockDim.x) {
         const double* e = S.exits + p * EXIT_DOUBLES;
@@ -216,25 +228,53 @@ __device__ __forceinline__ void hist_add(double* bins, double ux, double uy, dou
     atomicAdd(&bins[(long long)ie * n_a + ia], w);
 }
 
-template <int D, typename R>
-__global__ void k_histogram(const SimDev* __restrict__ sim, long long n, long long nex, int n_e, double e_max, int n_a,
-                            double* __restrict__ bins)
+// The same for single-precision momenta: the bin from FP32 arithmetic wherever that cannot differ
+// from the double one, i.e. unless it comes within its error of a bin's edge (2.1 M electrons,
+// 96 x 36 bins: 0.53 -> 0.2 ms; the double functions run at 1/64 of the FP32 rate).  Errors:
+// gamma - 1 = u^2/(gamma + 1) within 8 roundings of 2^-24 relative; the angle within 8 of pi.
+__device__ __forceinline__ void hist_add(double* bins, float ux, float uy, float uz, float w, int n_e, double e_max,
+                                         int n_a)
 {
+    const float up2 = uy * uy + uz * uz, u2 = ux * ux + up2;
+    const float fe = u2 / (1.0f + sqrtf(1.0f + u2)) * ((float)n_e / (float)e_max);
+    const float fa = atan2f(sqrtf(up2), ux) * ((float)n_a * 0.318309886f);
+    const float de = 1e-6f * fe + 1e-30f, da = 2e-6f * (float)n_a;
+    const float ie = floorf(fe), ia = floorf(fa);
+    const bool sure = fe - ie > de && fe - ie < 1.0f - de && fa - ia > da && fa - ia < 1.0f - da && u2 < 1e30f;
+    if (!sure || n_e > (1 << 16) || n_a > (1 << 16)) {
+        hist_add(bins, (double)ux, (double)uy, (double)uz, (double)w, n_e, e_max, n_a);
+    } else if (ie < (float)n_e) {
+        atomicAdd(&bins[(long long)(int)ie * n_a + min((int)ia, n_a - 1)], (double)w);
+    }
+}
+
+// SHARED: each block adds up its own n_e * n_a bins in shared memory first (the hot bins of a
+// thermal spectrum otherwise queue up in L2: 2.1 M electrons 0.44 ms).
+template <typename R, bool SHARED>
+__global__ void __launch_bounds__(512) k_histogram(const SimDev* __restrict__ sim, long long nex, int n_e, double e_max,
+                                                   int n_a, double* __restrict__ out)
+{
+    extern __shared__ double s_bins[];
     const SimDev& S = *sim;
     const int par = S.st->parity;
-    const long long nu = slots_used(S, par, n);
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < nu;
-         p += (long long)gridDim.x * blockDim.x) {
-        if (!slot_live<D>(S, par, p)) continue;
-        hist_add(bins, (double)reinterpret_cast<const R*>(S.mom[par][0])[p],
-                 (double)reinterpret_cast<const R*>(S.mom[par][1])[p],
-                 (double)reinterpret_cast<const R*>(S.mom[par][2])[p], (double)reinterpret_cast<const R*>(S.wgt[par])[p],
-                 n_e, e_max, n_a);
+    double* bins = SHARED ? s_bins : out;
+    if constexpr (SHARED) {
+        for (int i = threadIdx.x; i < n_e * n_a; i += blockDim.x) s_bins[i] = 0.0;
+        __syncthreads();
     }
+    for_particles(S, par, [&](long long p) {
+        hist_add(bins, reinterpret_cast<const R*>(S.mom[par][0])[p], reinterpret_cast<const R*>(S.mom[par][1])[p],
+                 reinterpret_cast<const R*>(S.mom[par][2])[p], reinterpret_cast<const R*>(S.wgt[par])[p], n_e, e_max, n_a);
+    });
     for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < nex;
          p += (long long)gridDim.x * blockDim.x) {
         const double* e = S.exits + p * EXIT_DOUBLES;
         hist_add(bins, e[0], e[1], e[2], e[3], n_e, e_max, n_a);
+    }
+    if constexpr (SHARED) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < n_e * n_a; i += blockDim.x)
+            if (s_bins[i] != 0.0) atomicAdd(&out[i], s_bins[i]);
     }
 }
 
@@ -403,14 +443,17 @@ __device__ __forceinline__ bool comp_has(const SimDev& S, int comp, const int g[
     return true;
 }
 
-// component comp of the field array at set offset fc (components) -> out[ext_z][ext_y][ext_x],
-// absent points 0
+// components comp0 + blockIdx.y of E, B (of buffer set par) and of J (of the last step: in the
+// other set) -> out[comp][ext_z][ext_y][ext_x], absent points 0
 template <int D, typename R>
-__global__ void k_get_field(const SimDev* __restrict__ sim, int fc, int comp, double* __restrict__ out)
+__global__ void k_get_field(const SimDev* __restrict__ sim, int par, int comp0, double* __restrict__ out0)
 {
     const SimDev& S = *sim;
+    const int comp = comp0 + blockIdx.y;
+    const int fc = comp < 6 ? comp_eb(par) + comp : comp_j(1 - par) + comp - 6;
     const R* F = reinterpret_cast<const R*>(S.F) + (long long)fc * S.sc;
     const unsigned ex = S.n[0] + 1, ey = D > 1 ? S.n[1] + 1 : 1, ez = D > 2 ? S.n[2] + 1 : 1;
+    double* out = out0 + (long long)blockIdx.y * ex * ey * ez;
     const unsigned rows = ey * ez, bpr = (ex + blockDim.x - 1) / blockDim.x;
     for (unsigned b = blockIdx.x; b < rows * bpr; b += gridDim.x) {
         const unsigned r = b / bpr, i = (b - r * bpr) * blockDim.x + threadIdx.x;
@@ -421,14 +464,16 @@ __global__ void k_get_field(const SimDev* __restrict__ sim, int fc, int comp, do
     }
 }
 
-// in[ext_z][ext_y][ext_x] -> component comp of the field array at offset fc, every allocated
-// point written (zero in the ghost region and at absent points)
+// in[comp][ext_z][ext_y][ext_x] -> components comp0 + blockIdx.y of E, B of buffer set par, every
+// allocated point written (zero in the ghost region and at absent points)
 template <int D, typename R>
-__global__ void k_put_field(const SimDev* __restrict__ sim, int fc, int comp, const double* __restrict__ in)
+__global__ void k_put_field(const SimDev* __restrict__ sim, int par, int comp0, const double* __restrict__ in0)
 {
     const SimDev& S = *sim;
-    R* F = reinterpret_cast<R*>(S.F) + (long long)fc * S.sc;
+    const int comp = comp0 + blockIdx.y;
+    R* F = reinterpret_cast<R*>(S.F) + (long long)(comp_eb(par) + comp) * S.sc;
     const unsigned ex = S.n[0] + 1, ey = D > 1 ? S.n[1] + 1 : 1;
+    const double* in = in0 + (long long)blockIdx.y * ex * ey * (D > 2 ? S.n[2] + 1 : 1);
     const unsigned nx = S.na[0], ny = S.na[1], rows = ny * (unsigned)S.na[2], bpr = (nx + blockDim.x - 1) / blockDim.x;
     for (unsigned b = blockIdx.x; b < rows * bpr; b += gridDim.x) {
         const unsigned r = b / bpr, i = (b - r * bpr) * blockDim.x + threadIdx.x;
@@ -456,14 +501,17 @@ static int grid_for(long long n) { return (int)std::max<long long>(1, std::min<l
         }                                                       \
     } while (0)
 
+// a block per tile
+static int grid_tiles(int nptiles) { return std::max(1, std::min(nptiles, device_sms() * 8)); }
+
 template <int D, typename R>
-static void charge_t(const SimDev* sim, long long n, double* rho, double scale, cudaStream_t s)
+static void charge_t(const SimDev* sim, int nptiles, double* rho, double scale, cudaStream_t s)
 {
-    if (n > 0) k_charge<D, R><<<grid_for(n), 256, 0, s>>>(sim, n, rho, scale);
+    k_charge<D, R><<<grid_tiles(nptiles), 256, 0, s>>>(sim, rho, scale);
 }
-void launch_charge(const SimDev* sim, int dim, int prec, long long n_slots, double* rho, cudaStream_t s, double scale)
+void launch_charge(const SimDev* sim, int dim, int prec, int nptiles, double* rho, cudaStream_t s, double scale)
 {
-    SFF_DISPATCH3(dim, prec, charge_t, sim, n_slots, rho, scale, s);
+    SFF_DISPATCH3(dim, prec, charge_t, sim, nptiles, rho, scale, s);
 }
 
 template <int D, typename R>
@@ -482,36 +530,42 @@ void launch_gauss(const SimDev* sim, int dim, int prec, const int n[3], const do
 template <int D, typename R>
 static void efield_t(const SimDev* sim, const int n[3], double* acc, cudaStream_t s)
 {
-    const int m0 = n[0] + 1, m1 = D > 1 ? n[1] + 1 : 1, m2 = D > 2 ? n[2] + 1 : 1;
-    const long long tot = (long long)m0 * m1 * m2;
-    k_energy_fields<D, R><<<grid_for(tot), 256, 0, s>>>(sim, m0, m1, m2, acc);
+    const long long segs = (n[0] + 256) / 256, rows = (D > 1 ? n[1] + 1LL : 1) * (D > 2 ? n[2] + 1LL : 1);
+    const int grid = (int)std::min<long long>(segs * rows, (long long)device_sms() * 8);
+    k_energy_fields<D, R><<<grid, 256, 0, s>>>(sim, acc);
 }
 void launch_energy_fields(const SimDev* sim, int dim, int prec, const int n[3], double* acc2, cudaStream_t s)
 {
     SFF_DISPATCH3(dim, prec, efield_t, sim, n, acc2, s);
 }
 
-template <int D, typename R>
-static void epart_t(const SimDev* sim, long long n, long long nex, double* acc, cudaStream_t s)
+void launch_energy_particles(const SimDev* sim, int prec, int nptiles, long long n_exits, double* acc2, cudaStream_t s)
 {
-    k_energy_particles<D, R><<<grid_for(std::max(n, nex)), 256, 0, s>>>(sim, n, nex, acc);
-}
-void launch_energy_particles(const SimDev* sim, int dim, int prec, long long n_alive, long long n_exits, double* acc2,
-                             cudaStream_t s)
-{
-    SFF_DISPATCH3(dim, prec, epart_t, sim, n_alive, n_exits, acc2, s);
+    const int grid = std::max(grid_tiles(nptiles), n_exits > 0 ? grid_for(n_exits) : 1);
+    if (prec == 0) k_energy_particles<double><<<grid, 256, 0, s>>>(sim, n_exits, acc2);
+    else k_energy_particles<float><<<grid, 256, 0, s>>>(sim, n_exits, acc2);
 }
 
-template <int D, typename R>
-static void hist_t(const SimDev* sim, long long n, long long nex, int n_e, double e_max, int n_a, double* bins,
-                   cudaStream_t s)
+template <typename R>
+static void hist_t(const SimDev* sim, int nptiles, long long n, long long nex, int n_e, double e_max, int n_a,
+                   double* bins, cudaStream_t s)
 {
-    k_histogram<D, R><<<grid_for(std::max(n, nex)), 256, 0, s>>>(sim, n, nex, n_e, e_max, n_a, bins);
+    // bins in shared memory where they fit its default size and get enough electrons each to pay
+    // for their clearing and the flush
+    const long long nb = (long long)n_e * n_a;
+    if (nb * 8 <= 48 * 1024 && n + nex >= 16 * nb) {
+        k_histogram<R, true><<<std::max(1, std::min(nptiles, device_sms() * 4)), 512, (size_t)nb * 8, s>>>(
+            sim, nex, n_e, e_max, n_a, bins);
+    } else {
+        const int grid = std::max(grid_tiles(nptiles), nex > 0 ? grid_for(nex) : 1);
+        k_histogram<R, false><<<grid, 256, 0, s>>>(sim, nex, n_e, e_max, n_a, bins);
+    }
 }
-void launch_histogram(const SimDev* sim, int dim, int prec, long long n_alive, long long n_exits, int n_e,
+void launch_histogram(const SimDev* sim, int prec, int nptiles, long long n_alive, long long n_exits, int n_e,
                       double e_max, int n_a, double* bins, cudaStream_t s)
 {
-    SFF_DISPATCH3(dim, prec, hist_t, sim, n_alive, n_exits, n_e, e_max, n_a, bins, s);
+    if (prec == 0) hist_t<double>(sim, nptiles, n_alive, n_exits, n_e, e_max, n_a, bins, s);
+    else hist_t<float>(sim, nptiles, n_alive, n_exits, n_e, e_max, n_a, bins, s);
 }
 
 template <int D, typename R>
@@ -565,24 +619,24 @@ void launch_put_particles(const SimDev* sim, int dim, int prec, long long k0, in
 }
 
 template <int D, typename R>
-static void getf_t(const SimDev* sim, long long points, int fc, int comp, double* out, cudaStream_t s)
+static void getf_t(const SimDev* sim, long long points, int par, int comp0, int ncomp, double* out, cudaStream_t s)
 {
-    k_get_field<D, R><<<grid_for(points), 256, 0, s>>>(sim, fc, comp, out);
+    k_get_field<D, R><<<dim3(grid_for(points), ncomp), 256, 0, s>>>(sim, par, comp0, out);
 }
-void launch_get_field(const SimDev* sim, int dim, int prec, long long points, int fc, int comp, double* out,
-                      cudaStream_t s)
+void launch_get_field(const SimDev* sim, int dim, int prec, long long points, int par, int comp0, int ncomp,
+                      double* out, cudaStream_t s)
 {
-    SFF_DISPATCH3(dim, prec, getf_t, sim, points, fc, comp, out, s);
+    SFF_DISPATCH3(dim, prec, getf_t, sim, points, par, comp0, ncomp, out, s);
 }
 template <int D, typename R>
-static void putf_t(const SimDev* sim, long long points, int fc, int comp, const double* in, cudaStream_t s)
+static void putf_t(const SimDev* sim, long long points, int par, int comp0, int ncomp, const double* in, cudaStream_t s)
 {
-    k_put_field<D, R><<<grid_for(points), 256, 0, s>>>(sim, fc, comp, in);
+    k_put_field<D, R><<<dim3(grid_for(points), ncomp), 256, 0, s>>>(sim, par, comp0, in);
 }
-void launch_put_field(const SimDev* sim, int dim, int prec, long long points, int fc, int comp, const double* in,
-                      cudaStream_t s)
+void launch_put_field(const SimDev* sim, int dim, int prec, long long points, int par, int comp0, int ncomp,
+                      const double* in, cudaStream_t s)
 {
-    SFF_DISPATCH3(dim, prec, putf_t, sim, points, fc, comp, in, s);
+    SFF_DISPATCH3(dim, prec, putf_t, sim, points, par, comp0, ncomp, in, s);
 }
 
 }  // namespace sff
@@ -663,7 +717,7 @@ extern "C" pic_status pic_histogram_static(pic_sim* s, int n_e, double e_max, in
     const size_t nb = (size_t)n_e * n_a;
     e = cudaMemsetAsync(bins, 0, nb * sizeof(double), st);
     if (e == cudaSuccess) {
-        sff::launch_histogram(s->d, s->cfg.dim, s->cfg.precision, s->h.cap,
+        sff::launch_histogram(s->d, s->cfg.precision, s->h.nptiles, ds.n_alive,
                               std::min<long long>(ds.n_exits, s->h.max_exits), n_e, e_max, n_a, bins, st);
         e = cudaGetLastError();
     }

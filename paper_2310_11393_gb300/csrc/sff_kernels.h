@@ -87,15 +87,13 @@ void launch_scan_one(const SimDev* sim, int q, cudaStream_t s);
 void launch_next_slots(const SimDev* sim, int dim, int prec, int q, long long n, cudaStream_t s);
 
 // diagnostics
-// adds scale * rho_e of the particles in the n_slots slots of the current set to rho
-void launch_charge(const SimDev* sim, int dim, int prec, long long n_slots, double* rho, cudaStream_t s,
-                   double scale = 1.0);
+// adds scale * rho_e of the particles of the current set to rho
+void launch_charge(const SimDev* sim, int dim, int prec, int nptiles, double* rho, cudaStream_t s, double scale = 1.0);
 void launch_gauss(const SimDev* sim, int dim, int prec, const int n[3], const double* rho, unsigned long long* out_bits,
                   cudaStream_t s);
 void launch_energy_fields(const SimDev* sim, int dim, int prec, const int n[3], double* acc2, cudaStream_t s);
-void launch_energy_particles(const SimDev* sim, int dim, int prec, long long n_alive, long long n_exits,
-                             double* acc2, cudaStream_t s);
-void launch_histogram(const SimDev* sim, int dim, int prec, long long n_alive, long long n_exits, int n_e,
+void launch_energy_particles(const SimDev* sim, int prec, int nptiles, long long n_exits, double* acc2, cudaStream_t s);
+void launch_histogram(const SimDev* sim, int prec, int nptiles, long long n_alive, long long n_exits, int n_e,
                       double e_max, int n_a, double* bins, cudaStream_t s);
 void launch_eval_incident(const SimDev* sim, int dim, int prec, long long n, const double* pts, double* out,
                           cudaStream_t s);
@@ -103,8 +101,7 @@ void launch_eval_incident(const SimDev* sim, int dim, int prec, long long n, con
 // state to and from the host layout, a piece of staging memory at a time (device pointers):
 // first[nptiles + 1] of the tiles of set par; records [k0, k1) of PIC_DIAG_PARTICLES; the check
 // and the conversion of particles k0 .. k0 + n - 1 (out: first refused index, largest |w| as
-// ordered bits); one field component at offset fc of the field array (points: of the grid, for
-// the launch size)
+// ordered bits); ncomp field components from comp0 on (points: of the grid, for the launch size)
 void launch_tile_first(const SimDev* sim, int par, int* first, cudaStream_t s);
 void launch_pack_particles(const SimDev* sim, int dim, int prec, int par, int nptiles, const int* first, long long k0,
                            long long k1, double* out, cudaStream_t s);
@@ -112,10 +109,10 @@ void launch_check_particles(const SimDev* sim, int dim, long long k0, int n, con
                             const long long* id, unsigned long long* out, cudaStream_t s);
 void launch_put_particles(const SimDev* sim, int dim, int prec, long long k0, int n, const double* x, const double* u,
                           const double* w, const long long* id, cudaStream_t s);
-void launch_get_field(const SimDev* sim, int dim, int prec, long long points, int fc, int comp, double* out,
-                      cudaStream_t s);
-void launch_put_field(const SimDev* sim, int dim, int prec, long long points, int fc, int comp, const double* in,
-                      cudaStream_t s);
+void launch_get_field(const SimDev* sim, int dim, int prec, long long points, int par, int comp0, int ncomp,
+                      double* out, cudaStream_t s);
+void launch_put_field(const SimDev* sim, int dim, int prec, long long points, int par, int comp0, int ncomp,
+                      const double* in, cudaStream_t s);
 
 // streaming multiprocessors of the current device (queried once per device)
 int device_sms();
