@@ -163,6 +163,7 @@ pic_status build_entry(const std::vector<pic_sim*>& sims, BatchEntry** out, std:
             g.inc_segs = std::max(g.inc_segs, (c.n[0] + 1 + 255) / 256);
             g.inc_rows = std::max(g.inc_rows, (c.dim > 1 ? c.n[1] + 1 : 1) * (c.dim > 2 ? c.n[2] + 1 : 1));
         }
+        g.tail = sff::step_has_tail(maxtiles);
         const int nsm = prop.multiProcessorCount;
         const int bp = std::max(1, sff::prepare_push(g.dim, g.prec, g.push_bx, g.push_by, psm));
         const int byy = std::max(1, sff::prepare_yee(g.dim, g.prec, ysm));
@@ -189,11 +190,15 @@ pic_status build_entry(const std::vector<pic_sim*>& sims, BatchEntry** out, std:
             return PIC_ECUDA;
         }
         // per group: push, then the tile scan (and cell sort) and the field solve
-        // concurrently, then the step end
+        // concurrently, then the step end (the last three in one launch where Group::tail)
         cudaError_t ce = cudaSuccess;
         for (auto& gr : e->groups) {
             sff::launch_incident_grid(gr.g, e->cs);
             sff::launch_push(gr.g, v == 1, e->cs);
+            if (gr.g.tail && v == 0) {
+                sff::launch_yee_tail(gr.g, e->cs);
+                continue;
+            }
             if (ce == cudaSuccess) ce = cudaEventRecord(e->ev_fork, e->cs);
             if (ce == cudaSuccess) ce = cudaStreamWaitEvent(e->cs2, e->ev_fork, 0);
             if (ce == cudaSuccess) {

@@ -4,6 +4,8 @@
 // diagnostics, explicit state I/O and batched stepping of many simulations.
 #include <cuda.h>
 #include <cuda_runtime.h>
+#include <sys/mman.h>
+#include <unistd.h>
 
 #include <algorithm>
 #include <atomic>
@@ -160,15 +162,22 @@ int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
 // bytes of the tiles' first-record table at the head of the staging memory
 size_t stage_head(int nptiles) { return align256((size_t)(nptiles + 1) * 4); }
 
-// Maps the pages of a host output buffer (one byte written per page, on several threads): a
-// copy into pages that are not mapped yet runs at the rate of one thread's page faults
-// (14-22 GB/s, mapped 190 GB/s).  The caller overwrites every byte.
+// Maps the pages of a host output buffer that are not mapped yet (one byte written per page, on
+// several threads): a copy into them runs at the rate of one thread's page faults (14-22 GB/s,
+// mapped 190 GB/s).  The caller overwrites every byte.
 void touch_pages(void* p, size_t bytes)
 {
-    const size_t page = 65536;       // the page size of the GPU's host; smaller pages: most faults
-    if (bytes < (1u << 20)) return;
-    host_parallel((long long)(bytes / page), 64, [=](long long a, long long b) {
-        for (long long k = a; k < b; ++k) static_cast<volatile char*>(p)[(size_t)k * page] = 0;
+    const size_t page = (size_t)sysconf(_SC_PAGESIZE);
+    const uintptr_t a = ((uintptr_t)p + page - 1) / page * page, e = (uintptr_t)p + bytes;
+    if (bytes < (1u << 20) || a >= e) return;
+    const size_t n = (e - a + page - 1) / page;      // pages that start inside the buffer
+    std::vector<unsigned char> in(n);
+    if (mincore((void*)a, e - a, in.data()) != 0) return;
+    size_t absent = 0;
+    for (unsigned char v : in) absent += !(v & 1);
+    if (absent < 16) return;
+    host_parallel((long long)n, 64, [=](long long i0, long long i1) {
+        for (long long k = i0; k < i1; ++k) *reinterpret_cast<volatile char*>(a + (size_t)k * page) = 0;
     });
 }
 int bits_for(int n)
@@ -504,26 +513,31 @@ void dev_free(pic_sim* s, void* p)
 }
 
 // One step as a CUDA graph; `sorted`: the variant whose particles are placed by cell.
-// After the push the graph forks: the tile scan (with, in the sorted variant, the cell-sort
-// placement) and the field solve touch disjoint data and run concurrently; the step end
-// joins them and numbers the next step's chunks (the graph starts at the push: see
-// ensure_prefix).
+// After the push come the tile scan (with, in the sorted variant, the cell-sort placement) and
+// the field solve, which touch disjoint data, and the step end, which numbers the next step's
+// chunks (the graph starts at the push: see ensure_prefix): one launch (step_has_tail), or a fork
+// of two branches that the step end joins.
 pic_status capture_step(pic_sim* s, bool sorted, GraphBundle* out)
 {
     cudaStream_t cs = s->cap_stream, cs2 = s->cap_stream2;
     CU_CHECK(s, cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     launch_incident_grid(s->grp, cs);
     launch_push(s->grp, sorted, cs);
-    cudaError_t e = cudaEventRecord(s->ev_fork, cs);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(cs2, s->ev_fork, 0);
-    if (e == cudaSuccess) {
-        launch_yee(s->grp, cs2);
-        e = cudaEventRecord(s->ev_join, cs2);
+    cudaError_t e = cudaSuccess;
+    if (s->grp.tail && !sorted) {
+        launch_yee_tail(s->grp, cs);
+    } else {
+        e = cudaEventRecord(s->ev_fork, cs);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(cs2, s->ev_fork, 0);
+        if (e == cudaSuccess) {
+            launch_yee(s->grp, cs2);
+            e = cudaEventRecord(s->ev_join, cs2);
+        }
+        launch_scan(s->grp, cs);
+        if (sorted) launch_cell_sort(s->grp, cs);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, s->ev_join, 0);
+        launch_step_end(s->grp, cs);
     }
-    launch_scan(s->grp, cs);
-    if (sorted) launch_cell_sort(s->grp, cs);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, s->ev_join, 0);
-    launch_step_end(s->grp, cs);
     cudaGraph_t g = nullptr;
     const cudaError_t ec = cudaStreamEndCapture(cs, &g);
     if (e == cudaSuccess) e = ec;
@@ -894,6 +908,7 @@ pic_status pic_init(const pic_config* cfg_in, const pic_allocator* alloc, void* 
     const int bs = std::max(1, scatter_blocks_per_sm(cfg->dim, cfg->precision));
     g.inc_any = h.incgrid;
     g.scan_blocks = h.nscanblk;
+    g.tail = step_has_tail(L.nptiles);
     g.cellscan_grid = std::max(1, std::min(L.nptiles, 8 * nsm));
     g.inc_segs = (cfg->n[0] + 1 + 255) / 256;
     g.inc_rows = (cfg->dim > 1 ? cfg->n[1] + 1 : 1) * (cfg->dim > 2 ? cfg->n[2] + 1 : 1);

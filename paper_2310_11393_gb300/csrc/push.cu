@@ -19,6 +19,7 @@
 #include <algorithm>
 
 #include "beam.cuh"
+#include "sched.cuh"
 #include "sff_common.cuh"
 #include "sff_kernels.h"
 
@@ -304,12 +305,10 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
     __syncthreads();
     unsigned phase = 0;
     int acq_sim = -1;         // thread 0: the simulation whose tensor maps it has acquired
-    for (;;) {
-        if (tid == 0) s_item = atomicAdd(counter, 1);
-        __syncthreads();
-        const int item = s_item;
-        __syncthreads();
-        if (item >= gprefix[nsims]) break;
+    // a block's first item is its own number, the following ones come from the counter
+    const int nitems = gprefix[nsims];
+    int item = blockIdx.x;
+    while (item < nitems) {
         const ChunkRef ck = ONE ? chunk_of_one(one, gprefix, item) : chunk_of(sims, nsims, gprefix, item);
         const SimDev& S = ONE ? one : sims[ck.sim];
         DevState* st = S.st;
@@ -735,10 +734,13 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
                 if (in) atomicAdd(&S.fcnt[nt], v);
             }
         }
-        if constexpr (sizeof(R) == 4) {
-            if (tid == 0) bulk_wait_read0();
+        if (nitems <= (int)gridDim.x) break;
+        if (tid == 0) {
+            s_item = gridDim.x + atomicAdd(counter, 1);
+            if constexpr (sizeof(R) == 4) bulk_wait_read0();
         }
         __syncthreads();
+        item = s_item;
     }
     if (tid == 0) bulk_wait0();
 }
@@ -757,94 +759,6 @@ __global__ void __launch_bounds__(push_threads<D, R>(), push_min_blocks<D, R>())
     k_push1(const __grid_constant__ SimDev one, const int* __restrict__ gprefix, int* __restrict__ counter, int sorting)
 {
     push_body<D, R, true, BX, BY>(nullptr, one, 1, gprefix, counter, sorting);
-}
-
-// Block-wide exclusive scan of one int per thread (blockDim a multiple of 32, <= 1024).
-__device__ __forceinline__ int block_exclusive_scan(int v, int* s_warp)
-{
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    int x = v;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, x, off);
-        if (lane >= off) x += y;
-    }
-    if (lane == 31) s_warp[wid] = x;
-    __syncthreads();
-    if (wid == 0) {
-        int w = lane < nw ? s_warp[lane] : 0;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, w, off);
-            if (lane >= off) w += y;
-        }
-        s_warp[lane] = w;
-    }
-    __syncthreads();
-    const int r = x - v + (wid > 0 ? s_warp[wid - 1] : 0);
-    __syncthreads();
-    return r;
-}
-
-// Chunks of tile t of buffer set q holding c particles from slot base: ctile / crange
-// entries from chunk index rc on.
-__device__ __forceinline__ void write_chunks(const SimDev& S, int q, int t, int base, int c, int rc)
-{
-    const int nc = (c + S.chunk - 1) / S.chunk;
-    for (int k = 0; k < nc; ++k) {
-        S.ctile[q][rc + k] = t;
-        const int a = base + k * S.chunk;
-        S.crange[q][rc + k] = make_int2(a, min(a + S.chunk, base + c));
-    }
-}
-
-// Tile scan of one simulation after a push into buffer set q (one block of 1024 threads):
-// per tile the particles now in set q (tcnt) and its frame count (fcnt) give
-//   set q:      tnum, the chunk offsets coff and the chunk map (ctile, crange) over the
-//               slots toff[q] set by the previous scan;
-//   set 1 - q:  toff = exclusive scan of tcnt + fcnt, the slots of the next step's push;
-// the particle total goes to n_next; the counts, cursors and frame counts are cleared.
-// `compact` (set-up): toff[q] = exclusive scan of tcnt first (no slack: the particles are
-// then placed there by the caller) and set 1 - q is left alone.
-__device__ void scan_counts(const SimDev& S, int q, bool compact)
-{
-    __shared__ int s_warp[32];
-    const int n = S.nptiles;
-    const int tid = threadIdx.x, nth = blockDim.x;
-    const int per = (n + nth - 1) / nth;
-    const int i0 = min(n, tid * per), i1 = min(n, i0 + per);
-    int lp = 0, lc = 0, lk = 0;
-    for (int i = i0; i < i1; ++i) {
-        const int c = S.tcnt[i];
-        lp += c;
-        lc += (c + S.chunk - 1) / S.chunk;
-        lk += c + S.fcnt[i];
-    }
-    int rp = block_exclusive_scan(lp, s_warp);
-    int rc = block_exclusive_scan(lc, s_warp);
-    int rk = block_exclusive_scan(lk, s_warp);
-    if (tid == nth - 1) atomicAdd(&S.st->n_next, rp + lp);
-    for (int i = i0; i < i1; ++i) {
-        const int c = S.tcnt[i];
-        if (compact) S.toff[q][i] = rp;
-        const int base = compact ? rp : S.toff[q][i];
-        S.tnum[q][i] = c;
-        S.coff[q][i] = rc;
-        write_chunks(S, q, i, base, c, rc);
-        if (!compact) S.toff[1 - q][i] = rk;
-        rp += c;
-        rc += (c + S.chunk - 1) / S.chunk;
-        rk += c + S.fcnt[i];
-        S.tcnt[i] = 0;
-        S.tcur[i] = 0;
-        S.fcnt[i] = 0;
-    }
-    if (tid == nth - 1) {
-        if (compact) S.toff[q][n] = rp;
-        else S.toff[1 - q][n] = rk;
-        S.coff[q][n] = rc;
-    }
-    __syncthreads();
 }
 
 __global__ void __launch_bounds__(1024) k_scan(const SimDev* __restrict__ sims)
@@ -1040,7 +954,7 @@ __global__ void __launch_bounds__(1024) k_prefix(const SimDev* __restrict__ sims
         r += sims[i].coff[sims[i].st->parity][sims[i].nptiles];
     }
     if (tid == nth - 1) gprefix[nsims] = r;
-    if (tid < 4) counters[tid] = 0;
+    if (tid < NCOUNTERS) counters[tid] = 0;
     if (nsims == 1) {
         const SimDev& S = sims[0];
         for (int j = tid; j < S.nscanblk; j += nth) S.scanflags[j] = 0ull;
@@ -1225,39 +1139,11 @@ __global__ void __launch_bounds__(256) k_cellscan(const SimDev* __restrict__ sim
     }
 }
 
-// Last node of every step: step counter, particle count and buffer parity of every
-// simulation of the group, then the next step's chunk numbering and work counters (what
-// k_prefix does), so that a step of the same group needs no k_prefix of its own.
+// Last node of a step whose tile scan and field solve are launches of their own.
 __global__ void __launch_bounds__(1024) k_step_end(const SimDev* __restrict__ sims, int nsims,
                                                    int* __restrict__ gprefix, int* __restrict__ counters)
 {
-    __shared__ int s_warp[32];
-    const int tid = threadIdx.x, nth = blockDim.x;
-    const int per = (nsims + nth - 1) / nth;
-    const int i0 = min(nsims, tid * per), i1 = min(nsims, i0 + per);
-    int l = 0;
-    for (int i = i0; i < i1; ++i) {
-        const SimDev& S = sims[i];
-        DevState* st = S.st;
-        const int np = 1 - st->parity;
-        st->n_alive = st->n_next;
-        st->n_next = 0;
-        st->parity = np;
-        st->step += 1;
-        l += S.coff[np][S.nptiles];
-    }
-    int r = block_exclusive_scan(l, s_warp);
-    for (int i = i0; i < i1; ++i) {
-        gprefix[i] = r;
-        r += sims[i].coff[sims[i].st->parity][sims[i].nptiles];   // the parity this thread just set
-    }
-    if (tid == nth - 1) gprefix[nsims] = r;
-    if (tid < 4) counters[tid] = 0;
-    if (nsims == 1) {
-        const SimDev& S = sims[0];
-        for (int j = tid; j < S.nscanblk; j += nth) S.scanflags[j] = 0ull;
-        if (tid == 0) *S.scanticket = 0;
-    }
+    end_step(sims, nsims, gprefix, counters);
 }
 
 // Incident field on the Yee nodes (the prescribed-field route): one block per row segment of

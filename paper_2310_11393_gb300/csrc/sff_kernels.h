@@ -19,6 +19,8 @@ constexpr int COMP_TOTAL = 18, NFCOMP_INC = 24;
 __host__ __device__ constexpr int comp_eb(int parity) { return 6 * parity; }
 __host__ __device__ constexpr int comp_j(int parity) { return 12 + 3 * parity; }
 
+constexpr int NCOUNTERS = 5;
+
 // One launch group: simulations of one dimension and precision advanced together.
 // Particles are processed in chunks of at most SimDev::chunk particles of one tile; the
 // chunks of all simulations of the group are numbered 0 .. gprefix[nsims)-1 each step.
@@ -28,12 +30,13 @@ struct Group {
     int* gprefix;          // device [nsims + 1]: first global chunk of each simulation
     const Work* ywork;     // field-solver tiles, device
     int nywork;
-    int* counters;         // device: [0] push, [1] scatter, [2] field solver
+    int* counters;         // device: [0] push, [1] scatter, [2] field solver, [3] cell count, [4] blocks done
     int dim, prec;
     size_t push_smem, yee_smem;
     int push_bx, push_by;  // row pitch and rows per plane of the push box (0: they differ between members)
     int push_grid, yee_grid, scatter_grid;
     int inc_any, inc_segs, inc_rows;   // incident field on the grid: any member, x segments, rows
+    int tail;                          // the field solver's launch takes the tile scan and the step end along
     int scan_blocks;                   // single simulation: blocks of the multi-block tile scan
     int cellscan_grid;                 // cell sort: blocks per simulation of the per-tile cell scan
     const SimDev* one;                 // single simulation: its host descriptor, passed by value to the
@@ -71,6 +74,7 @@ void launch_scan(const Group& g, cudaStream_t s);
 // the members that have a cell sort (after launch_push(.., true, ..) and the tile scan)
 void launch_cell_sort(const Group& g, cudaStream_t s);
 void launch_yee(const Group& g, cudaStream_t s);
+void launch_yee_tail(const Group& g, cudaStream_t s);      // field solve, tile scan and step end (Group::tail)
 void launch_step_end(const Group& g, cudaStream_t s);
 void launch_incident_grid(const Group& g, cudaStream_t s);
 
@@ -116,6 +120,12 @@ void launch_put_field(const SimDev* sim, int dim, int prec, long long points, in
 
 // streaming multiprocessors of the current device (queried once per device)
 int device_sms();
+
+// Do the tile scan (one block per simulation) and the step end ride on the field solver's launch?
+// They save two launches and a fork of the step graph, some 4 us of a step; one block scans 4096
+// tiles in about 10 us beside a field solve of at least that size.  Larger simulations scan over
+// several blocks in a launch of their own.
+inline bool step_has_tail(int nptiles) { return nptiles <= 4096; }
 
 // Is field-solver tile t a work item?  In 2D and 3D a tile (column) whose first point lies on
 // the node line / plane x = n_x (or y = n_y), which holds nothing else, is not: the one before

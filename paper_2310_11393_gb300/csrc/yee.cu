@@ -21,6 +21,7 @@
 #include <type_traits>
 
 #include "beam.cuh"
+#include "sched.cuh"
 #include "sff_common.cuh"
 #include "sff_kernels.h"
 
@@ -57,7 +58,7 @@ __device__ __forceinline__ bool has_point(const SimDev& S, int comp, const int g
 // with no acquire); otherwise the descriptors are read from the device array `sims`.
 template <int D, typename R, int TX, int TY, int TZ, bool ONE>
 __device__ __forceinline__ void yee_body(const SimDev* __restrict__ sims, const SimDev& one,
-                                         const Work* __restrict__ work, int nwork, int* __restrict__ counter)
+                                         const Work* __restrict__ work, int nwork, int* __restrict__ counter, int nscan)
 {
     constexpr int HX = 4, HY = D > 1 ? 2 : 0, HZ = D > 2 ? 2 : 0;
     constexpr int EX = TX + 2 * HX, EY = TY + 2 * HY, EZ = TZ + 2 * HZ;
@@ -80,8 +81,12 @@ __device__ __forceinline__ void yee_body(const SimDev* __restrict__ sims, const 
     R* Out = reinterpret_cast<R*>(smem_raw + OOFF);    // [6][TZ][TY][TX]
     // Two box buffers: while a block computes one tile, the TMA loads of its next tile (taken
     // from the work counter one tile ahead) land in the other.
+    // a block's first item is its number among the solving blocks, the following ones come from
+    // the counter (and there are none when every item has a block of its own)
+    const int nblk = (int)gridDim.x - nscan;
     auto fetch = [&]() {
-        if (tid == 0) s_item = atomicAdd(counter, 1);
+        if (nwork <= nblk) return nwork;
+        if (tid == 0) s_item = nblk + atomicAdd(counter, 1);
         __syncthreads();
         const int it = s_item;
         __syncthreads();
@@ -119,7 +124,7 @@ __device__ __forceinline__ void yee_body(const SimDev* __restrict__ sims, const 
         tma_load_box<D>(box, &S.tm_yin, o, comp_eb(p), &bars[b]);
         tma_load_box<D>(box + JOFF, &S.tm_yj, o, comp_j(p), &bars[b]);
     };
-    int item = fetch();
+    int item = (int)blockIdx.x - nscan;
     if (item < nwork) issue(item, 0);
     int buf = 0;
     while (item < nwork) {
@@ -316,16 +321,18 @@ __device__ __forceinline__ void yee_body(const SimDev* __restrict__ sims, const 
 
 template <int D, typename R, int TX, int TY, int TZ>
 __global__ void __launch_bounds__(256) k_yee(const SimDev* __restrict__ sims, const Work* __restrict__ work,
-                                             int nwork, int* __restrict__ counter)
+                                             int nwork, int* __restrict__ counter, const StepTail tail)
 {
-    yee_body<D, R, TX, TY, TZ, false>(sims, *sims, work, nwork, counter);
+    if (!tail_scan(tail)) yee_body<D, R, TX, TY, TZ, false>(sims, *sims, work, nwork, counter, tail.nscan);
+    tail_end(tail);
 }
 
 template <int D, typename R, int TX, int TY, int TZ>
 __global__ void __launch_bounds__(256) k_yee1(const __grid_constant__ SimDev one, const Work* __restrict__ work,
-                                              int nwork, int* __restrict__ counter)
+                                              int nwork, int* __restrict__ counter, const StepTail tail)
 {
-    yee_body<D, R, TX, TY, TZ, true>(nullptr, one, work, nwork, counter);
+    if (!tail_scan(tail)) yee_body<D, R, TX, TY, TZ, true>(nullptr, one, work, nwork, counter, tail.nscan);
+    tail_end(tail);
 }
 
 // ---------------------------------------------------------------------------------
@@ -346,7 +353,7 @@ __global__ void __launch_bounds__(256) k_yee1(const __grid_constant__ SimDev one
 // ---------------------------------------------------------------------------------
 template <typename R, int PY, int NT, bool ONE>
 __device__ __forceinline__ void yee2r_body(const SimDev* __restrict__ sims, const SimDev& one,
-                                           const Work* __restrict__ work, int nwork, int* __restrict__ counter)
+                                           const Work* __restrict__ work, int nwork, int* __restrict__ counter, int nscan)
 {
     constexpr int PX = 32;
     constexpr int BX = PX + 8, BY = PY + 4, BV = BX * BY, TV = PX * PY;
@@ -397,8 +404,12 @@ __device__ __forceinline__ void yee2r_body(const SimDev* __restrict__ sims, cons
         pN = has && lx >= 3 && ly >= 1;
         po = (has && lx >= 4 && lx < PX + 4 && ly >= 2 && ly < PY + 2) ? (lx - 4) + PX * (ly - 2) : -1;
     }
+    // a block's first item is its number among the solving blocks, the following ones come from
+    // the counter (and there are none when every item has a block of its own)
+    const int nblk = (int)gridDim.x - nscan;
     auto fetch = [&]() {
-        if (tid == 0) s_item = atomicAdd(counter, 1);
+        if (nwork <= nblk) return nwork;
+        if (tid == 0) s_item = nblk + atomicAdd(counter, 1);
         __syncthreads();
         const int it = s_item;
         __syncthreads();
@@ -423,7 +434,7 @@ __device__ __forceinline__ void yee2r_body(const SimDev* __restrict__ sims, cons
         tma_load_box<2>(box, &S.tm_yin, o, comp_eb(p), &bars[b]);
         tma_load_box<2>(box + JOFF, &S.tm_yj, o, comp_j(p), &bars[b]);
     };
-    int item = fetch();
+    int item = (int)blockIdx.x - nscan;
     if (item < nwork) issue(item, 0);
     int buf = 0;
     while (item < nwork) {
@@ -559,16 +570,18 @@ __device__ __forceinline__ void yee2r_body(const SimDev* __restrict__ sims, cons
 
 template <typename R, int PY, int NT>
 __global__ void __launch_bounds__(NT, 2) k_yee2r(const SimDev* __restrict__ sims, const Work* __restrict__ work,
-                                                 int nwork, int* __restrict__ counter)
+                                                 int nwork, int* __restrict__ counter, const StepTail tail)
 {
-    yee2r_body<R, PY, NT, false>(sims, *sims, work, nwork, counter);
+    if (!tail_scan(tail)) yee2r_body<R, PY, NT, false>(sims, *sims, work, nwork, counter, tail.nscan);
+    tail_end(tail);
 }
 
 template <typename R, int PY, int NT>
 __global__ void __launch_bounds__(NT, 2) k_yee2r1(const __grid_constant__ SimDev one, const Work* __restrict__ work,
-                                                  int nwork, int* __restrict__ counter)
+                                                  int nwork, int* __restrict__ counter, const StepTail tail)
 {
-    yee2r_body<R, PY, NT, true>(nullptr, one, work, nwork, counter);
+    if (!tail_scan(tail)) yee2r_body<R, PY, NT, true>(nullptr, one, work, nwork, counter, tail.nscan);
+    tail_end(tail);
 }
 
 // ---------------------------------------------------------------------------------
@@ -597,7 +610,7 @@ __global__ void __launch_bounds__(NT, 2) k_yee2r1(const __grid_constant__ SimDev
 // ---------------------------------------------------------------------------------
 template <typename R, int PX, int PY, int NS, int NT, bool ONE>
 __device__ __forceinline__ void yee3s_body(const SimDev* __restrict__ sims, const SimDev& one,
-                                           const Work* __restrict__ work, int nwork, int* __restrict__ counter)
+                                           const Work* __restrict__ work, int nwork, int* __restrict__ counter, int nscan)
 {
     constexpr int TV = PX * PY;
     constexpr int BX = PX + 8, BY = PY + 4, BV = BX * BY;
@@ -655,12 +668,9 @@ __device__ __forceinline__ void yee3s_body(const SimDev* __restrict__ sims, cons
         po = (has && lx >= 4 && lx < PX + 4 && ly >= 2 && ly < PY + 2) ? (lx - 4) + PX * (ly - 2) : -1;
     }
     uint32_t ph = 0;      // mbarrier phase of each stage
-    for (;;) {
-        if (tid == 0) s_item = atomicAdd(counter, 1);
-        __syncthreads();
-        const int item = s_item;
-        __syncthreads();
-        if (item >= nwork) break;
+    const int nblk = (int)gridDim.x - nscan;
+    // (first item: the block's number among the solving blocks; then from the counter)
+    for (int item = (int)blockIdx.x - nscan; item < nwork;) {
         const Work wk = work[item];
         const SimDev& S = ONE ? one : sims[wk.sim];
         DevState* st = S.st;
@@ -992,22 +1002,29 @@ __device__ __forceinline__ void yee3s_body(const SimDev* __restrict__ sims, cons
             }
             return;
         }
+        if (nwork <= nblk) break;
+        if (tid == 0) s_item = nblk + atomicAdd(counter, 1);
+        __syncthreads();
+        item = s_item;
+        __syncthreads();
     }
     if (tid == 0) bulk_wait0();
 }
 
 template <typename R, int PX, int PY, int NS, int NT>
 __global__ void __launch_bounds__(NT) k_yee3s(const SimDev* __restrict__ sims, const Work* __restrict__ work,
-                                              int nwork, int* __restrict__ counter)
+                                              int nwork, int* __restrict__ counter, const StepTail tail)
 {
-    yee3s_body<R, PX, PY, NS, NT, false>(sims, *sims, work, nwork, counter);
+    if (!tail_scan(tail)) yee3s_body<R, PX, PY, NS, NT, false>(sims, *sims, work, nwork, counter, tail.nscan);
+    tail_end(tail);
 }
 
 template <typename R, int PX, int PY, int NS, int NT>
 __global__ void __launch_bounds__(NT) k_yee3s1(const __grid_constant__ SimDev one, const Work* __restrict__ work,
-                                               int nwork, int* __restrict__ counter)
+                                               int nwork, int* __restrict__ counter, const StepTail tail)
 {
-    yee3s_body<R, PX, PY, NS, NT, true>(nullptr, one, work, nwork, counter);
+    if (!tail_scan(tail)) yee3s_body<R, PX, PY, NS, NT, true>(nullptr, one, work, nwork, counter, tail.nscan);
+    tail_end(tail);
 }
 
 // 1D field-solver tiles (must match the host's tile choice)
@@ -1019,27 +1036,28 @@ struct YeeTile<1> {
 };
 
 template <int D, typename R>
-static void yee_t(const Group& g, cudaStream_t s)
+static void yee_t(const Group& g, bool with_tail, cudaStream_t s)
 {
+    const StepTail tail = {g.sims, g.nsims, with_tail ? g.nsims : 0, g.gprefix, g.counters};
     if constexpr (D == 3) {
         if (g.one)
             k_yee3s1<R, Y3_PX, Y3_PY, Y3_NS, Y3_NT>
-                <<<g.yee_grid, Y3_NT, g.yee_smem, s>>>(*g.one, g.ywork, g.nywork, g.counters + 2);
+                <<<g.yee_grid + tail.nscan, Y3_NT, g.yee_smem, s>>>(*g.one, g.ywork, g.nywork, g.counters + 2, tail);
         else
             k_yee3s<R, Y3_PX, Y3_PY, Y3_NS, Y3_NT>
-                <<<g.yee_grid, Y3_NT, g.yee_smem, s>>>(g.sims, g.ywork, g.nywork, g.counters + 2);
+                <<<g.yee_grid + tail.nscan, Y3_NT, g.yee_smem, s>>>(g.sims, g.ywork, g.nywork, g.counters + 2, tail);
     } else if constexpr (D == 2) {
         if (g.one)
-            k_yee2r1<R, Y2_PY, Y2_NT><<<g.yee_grid, Y2_NT, g.yee_smem, s>>>(*g.one, g.ywork, g.nywork, g.counters + 2);
+            k_yee2r1<R, Y2_PY, Y2_NT><<<g.yee_grid + tail.nscan, Y2_NT, g.yee_smem, s>>>(*g.one, g.ywork, g.nywork, g.counters + 2, tail);
         else
-            k_yee2r<R, Y2_PY, Y2_NT><<<g.yee_grid, Y2_NT, g.yee_smem, s>>>(g.sims, g.ywork, g.nywork, g.counters + 2);
+            k_yee2r<R, Y2_PY, Y2_NT><<<g.yee_grid + tail.nscan, Y2_NT, g.yee_smem, s>>>(g.sims, g.ywork, g.nywork, g.counters + 2, tail);
     } else {
         if (g.one)
             k_yee1<D, R, YeeTile<D>::X, YeeTile<D>::Y, YeeTile<D>::Z>
-                <<<g.yee_grid, 256, g.yee_smem, s>>>(*g.one, g.ywork, g.nywork, g.counters + 2);
+                <<<g.yee_grid + tail.nscan, 256, g.yee_smem, s>>>(*g.one, g.ywork, g.nywork, g.counters + 2, tail);
         else
             k_yee<D, R, YeeTile<D>::X, YeeTile<D>::Y, YeeTile<D>::Z>
-                <<<g.yee_grid, 256, g.yee_smem, s>>>(g.sims, g.ywork, g.nywork, g.counters + 2);
+                <<<g.yee_grid + tail.nscan, 256, g.yee_smem, s>>>(g.sims, g.ywork, g.nywork, g.counters + 2, tail);
     }
 }
 
@@ -1091,7 +1109,8 @@ static void attr_yee(size_t smem, int* out)
         }                                                       \
     } while (0)
 
-void launch_yee(const Group& g, cudaStream_t s) { SFF_DISPATCH2(g.dim, g.prec, yee_t, g, s); }
+void launch_yee(const Group& g, cudaStream_t s) { SFF_DISPATCH2(g.dim, g.prec, yee_t, g, false, s); }
+void launch_yee_tail(const Group& g, cudaStream_t s) { SFF_DISPATCH2(g.dim, g.prec, yee_t, g, true, s); }
 
 int prepare_yee(int dim, int prec, size_t smem)
 {
