@@ -517,16 +517,24 @@ void dev_free(pic_sim* s, void* p)
 // the field solve, which touch disjoint data, and the step end, which numbers the next step's
 // chunks (the graph starts at the push: see ensure_prefix): one launch (step_has_tail), or a fork
 // of two branches that the step end joins.
-pic_status capture_step(pic_sim* s, bool sorted, GraphBundle* out)
+//
+// `steps` of them in one graph (steps with a tail only): the edge between two kernels of a graph
+// is shorter than that between two graphs.
+constexpr int MANY_STEPS = 16;
+pic_status capture_step(pic_sim* s, bool sorted, int steps, GraphBundle* out)
 {
     cudaStream_t cs = s->cap_stream, cs2 = s->cap_stream2;
     CU_CHECK(s, cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-    launch_incident_grid(s->grp, cs);
-    launch_push(s->grp, sorted, cs);
     cudaError_t e = cudaSuccess;
     if (s->grp.tail && !sorted) {
-        launch_yee_tail(s->grp, cs);
+        for (int k = 0; k < steps; ++k) {
+            launch_incident_grid(s->grp, cs);
+            launch_push(s->grp, sorted, cs);
+            launch_yee_tail(s->grp, cs);
+        }
     } else {
+        launch_incident_grid(s->grp, cs);
+        launch_push(s->grp, sorted, cs);
         e = cudaEventRecord(s->ev_fork, cs);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(cs2, s->ev_fork, 0);
         if (e == cudaSuccess) {
@@ -919,8 +927,8 @@ pic_status pic_init(const pic_config* cfg_in, const pic_allocator* alloc, void* 
     INIT_CHECK(cudaStreamCreateWithFlags(&s->cap_stream2, cudaStreamNonBlocking));
     INIT_CHECK(cudaEventCreateWithFlags(&s->ev_fork, cudaEventDisableTiming));
     INIT_CHECK(cudaEventCreateWithFlags(&s->ev_join, cudaEventDisableTiming));
-    if ((r = capture_step(s, false, &s->step_graph)) != PIC_OK) return cleanup(r);
-    if (s->sort_every > 0 && (r = capture_step(s, true, &s->sort_graph)) != PIC_OK) return cleanup(r);
+    if ((r = capture_step(s, false, 1, &s->step_graph)) != PIC_OK) return cleanup(r);
+    if (s->sort_every > 0 && (r = capture_step(s, true, 1, &s->sort_graph)) != PIC_OK) return cleanup(r);
 #undef INIT_CHECK
     *out = s;
     return PIC_OK;
@@ -932,7 +940,19 @@ pic_status pic_step(pic_sim* s, int n_steps, void* stream)
     if (n_steps < 0) return fail(s, PIC_EINVAL, "n_steps < 0");
     cudaStream_t st = (cudaStream_t)stream;
     if (n_steps > 0) ensure_prefix(s, st);
-    for (int i = 0; i < n_steps; ++i)
+    int i = 0;
+    if (s->grp.tail && s->sort_every <= 0 && n_steps >= 4 * MANY_STEPS) {
+        // (not while the caller captures the stream: only its launches belong there)
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        CU_CHECK(s, cudaStreamIsCapturing(st, &cap));
+        if (!s->many_graph.exec && cap == cudaStreamCaptureStatusNone) {
+            const pic_status r = capture_step(s, false, MANY_STEPS, &s->many_graph);
+            if (r != PIC_OK) return r;
+        }
+        if (s->many_graph.exec)
+            for (; i + MANY_STEPS <= n_steps; i += MANY_STEPS) CU_CHECK(s, cudaGraphLaunch(s->many_graph.exec, st));
+    }
+    for (; i < n_steps; ++i)
         CU_CHECK(s, cudaGraphLaunch(next_is_sort(s) ? s->sort_graph.exec : s->step_graph.exec, st));
     return PIC_OK;
 }
@@ -982,6 +1002,8 @@ pic_status pic_destroy(pic_sim* s)
     batch_forget(s);
     if (s->step_graph.exec) cudaGraphExecDestroy(s->step_graph.exec);
     if (s->step_graph.graph) cudaGraphDestroy(s->step_graph.graph);
+    if (s->many_graph.exec) cudaGraphExecDestroy(s->many_graph.exec);
+    if (s->many_graph.graph) cudaGraphDestroy(s->many_graph.graph);
     if (s->sort_graph.exec) cudaGraphExecDestroy(s->sort_graph.exec);
     if (s->sort_graph.graph) cudaGraphDestroy(s->sort_graph.graph);
     if (s->cap_stream) cudaStreamDestroy(s->cap_stream);

@@ -50,6 +50,7 @@ struct pic_sim {
     double* d_acc = nullptr;     // 8 doubles
     unsigned long long* d_bits = nullptr;
     GraphBundle step_graph;
+    GraphBundle many_graph;      // MANY_STEPS steps (captured when a call first asks for a few times that)
     // id of the launch group whose chunk numbering and work counters are set for this sim's
     // current particle layout (each step ends by setting them for its own group; any other
     // change of the layout clears it, and the next step of a group starts with k_prefix)
