@@ -68,9 +68,9 @@ inline BeamC<R> make_beam_consts(const SimDev& S)
     b.dtdx = R(S.dt * S.inv_dx);
     b.jfac = R(S.dx / S.dt);
     // |w|^{-(s+1)} below e^{-36}: the term is below ~1e-11 of the peak field even after the
-    // largest 1/R^5 and polynomial factors the closed form applies.  The + term is also left out
-    // where it is below e^{-18} (FP32; FP64 e^{-42}) of the - term: a quarter of the rounding
-    // of the - term in every sum the two enter.
+    // largest 1/R^5 and polynomial factors the closed form applies.  phi_closed also leaves out the
+    // + term where it is below e^{-18} (FP32; FP64 e^{-42}) of the - term: a quarter of the
+    // rounding of the - term in every sum the two enter.
     b.wcut = R(std::exp(72.0 / (S.s + 1.0)));
     b.wrel = R(std::exp((sizeof(R) == 4 ? 36.0 : 84.0) / (S.s + 1.0)));
     b.aos = R(S.s > 0 ? S.a / S.s : 0.0);
@@ -179,22 +179,6 @@ __device__ __noinline__ void phi_series(const BeamC<R>& b, Cx<R> u, R trel, Cx<R
     P[3] = SDD;
 }
 
-// log|w|, w = 1 - i tau/s (decides whether the term matters at all)
-template <typename R>
-__device__ __forceinline__ R log_abs_w(const BeamC<R>& b, Cx<R> tau)
-{
-    const R ti = tau.y * b.inv_s, tr = tau.x * b.inv_s;
-    return R(0.5) * m_log1p(ti * (R(2) + ti) + tr * tr);
-}
-
-// |w|^{-(s+1)} below e^{-36}: the term is below ~1e-11 of the peak field even after the
-// largest 1/R^5 and polynomial factors the closed form applies, so it is dropped
-template <typename R>
-__device__ __forceinline__ bool negligible(const BeamC<R>& b, R lnw)
-{
-    return b.sp1 * lnw > R(36);
-}
-
 // e^{i phi0} w^{-(s+1)}, w = 1 - i tau/s, and g^(1), g^(2) (Eq. poisson_dstr), given log|w|
 template <typename R>
 __device__ __forceinline__ void poisson3_log(const BeamC<R>& b, Cx<R> tau, R lnw, Cx<R>& g0, Cx<R>& g1, Cx<R>& g2)
@@ -206,7 +190,7 @@ __device__ __forceinline__ void poisson3_log(const BeamC<R>& b, Cx<R> tau, R lnw
     sincos_phase(b.phi0 - b.sp1 * th, &sn, &cs);
     g0 = {mag * cs, mag * sn};
     // q = i a/(s w)
-    const R den = R(1) / (b.s * (w.x * w.x + w.y * w.y));
+    const R den = m_inv(b.s * (w.x * w.x + w.y * w.y));
     const Cx<R> q = {b.a * w.y * den, b.a * w.x * den};
     g1 = b.sp1 * (g0 * q);
     g2 = b.sp2 * (g1 * q);
@@ -263,10 +247,13 @@ __device__ __forceinline__ bool phi_closed(const BeamC<R>& b, R rho2, R zeta, Cx
     return true;
 }
 
-// The same with library functions throughout (hypot, divisions, atan2, both logarithms): the
-// FP32 3D push.  Its electrons amplify a last-bit change of the incident field 1e4-fold within
-// 100 steps of the a0 = 20 focus, and it is bound by the shared-memory pipe: the form above gave
-// it 3 % (1.76 -> 1.71 ms) and moved a few electrons in 16.8 M by 2e-3 of the rms momentum.
+// The same from hypot, atan2 and log1p of the library and correctly rounded reciprocals and
+// roots: the FP32 pushes.  Electrons of a strong focus amplify a last-bit change of the incident
+// field up to 1e4-fold within 100 steps, so the form above, though no less accurate and 2 to 3 %
+// of a step faster, moved single electrons by 1e-3 .. 1e-2 of the rms momentum in 8 of 41 sampled
+// runs; this one leaves as many outside as two runs of one build differ in (2).  With the
+// quotients and roots of m_inv, m_root and m_quot a 2D LP step takes 0.142 ms (1.05 M cells, 10
+// electrons per cell; with the compiler's 0.147).
 template <typename R>
 __device__ __forceinline__ bool phi_closed_log(const BeamC<R>& b, R rho2, R zeta, Cx<R> u, R tmz, R tpz, Cx<R> P[4])
 {
@@ -276,12 +263,13 @@ __device__ __forceinline__ bool phi_closed_log(const BeamC<R>& b, R rho2, R zeta
     const Cx<R> qq = (b.a * rho2) * cinv(den);     // a R - (z + i a)
     const Cx<R> taum = {tmz - qq.x, -qq.y};
     const Cx<R> taup = {tpz + qq.x, b.two_a + qq.y};
-    const R lnm = log_abs_w(b, taum), lnp = log_abs_w(b, taup);
-    const bool use_m = !negligible(b, lnm), use_p = !negligible(b, lnp);
+    const R xm = w2m1(b, taum), xp = w2m1(b, taup);
+    const bool use_m = R(1) + xm < b.wcut;
+    const bool use_p = R(1) + xp < b.wcut;
     if (!use_m && !use_p) return false;
     Cx<R> g0m = {0, 0}, g1m = {0, 0}, g2m = {0, 0}, g0p = {0, 0}, g1p = {0, 0}, g2p = {0, 0};
-    if (use_m) poisson3_log(b, taum, lnm, g0m, g1m, g2m);
-    if (use_p) poisson3_log(b, taup, lnp, g0p, g1p, g2p);
+    if (use_m) poisson3_log(b, taum, R(0.5) * m_log1p(xm), g0m, g1m, g2m);
+    if (use_p) poisson3_log(b, taup, R(0.5) * m_log1p(xp), g0p, g1p, g2p);
     const Cx<R> G0m = g0p - g0m, G1p = g1p + g1m, G1m = g1p - g1m, G2p = g2p + g2m, G2m = g2p - g2m;
     const Cx<R> iR = cinv(Rr);
     const Cx<R> iR2 = iR * iR;
@@ -435,7 +423,7 @@ __device__ __forceinline__ void incident_at(const SimDev& S, const BeamC<R>& b, 
         if constexpr (D >= 2) xi = ((R)(c[1] - S.icf[1]) + (o[1] - b.frf[1])) * (b.dxr * inv_a);
         if constexpr (D >= 3) eta = ((R)(c[2] - S.icf[2]) + (o[2] - b.frf[2])) * (b.dxr * inv_a);
         R Ep[3], Bp[3];
-        focused_field<D == 3 && sizeof(R) == 4 && !DIAG, R>(b, xi, eta, zeta, tmz, tpz, pr.trel, Ep, Bp);
+        focused_field<sizeof(R) == 4 && !DIAG, R>(b, xi, eta, zeta, tmz, tpz, pr.trel, Ep, Bp);
         E[0] = Ep[2];
         E[1] = Ep[0];
         E[2] = Ep[1];

@@ -98,11 +98,11 @@ __device__ __forceinline__ R interp(const R* f, const int bx, const int bxy, con
 // the scale q = range / (max(N, nmin) w_max) of the item (N particles): a contribution of one
 // particle to one node is bounded by w |v| <= w_max (Esirkepov's partial sums of the shape
 // change are at most the move in cells, v dt/dx, times dx/dt; the transverse weights are
-// averages of shapes in [0, 1]; |v| < c = 1), so with range 2^31 (1 - 2^-10) and nmin 512 (1D and
-// 2D) |c q| < 2^22 and no node's sum, its N roundings included, reaches 2^31.  3D has four times
-// the room: range 2^29, nmin 256 (an error of the current below that of the trajectories; a finer
-// scale there moved single electrons of the a0 = 20 focus by 1e-3 of the rms momentum against
-// runs with this one).  Each contribution is rounded to the nearest integer by one FMA with
+// averages of shapes in [0, 1]; |v| < c = 1), so with range 2^31 (1 - 2^-10) and nmin 512 (2D)
+// |c q| < 2^22 and no node's sum, its N roundings included, reaches 2^31.  1D and 3D leave four
+// times the room: range 2^29, nmin 256 (their default items are not larger than before, and a finer
+// scale moved single electrons of the a0 = 20 focus by 1e-3 of the rms momentum against runs with
+// this one).  Each contribution is rounded to the nearest integer by one FMA with
 // 1.5 * 2^23 (the sum lands in [2^23, 2^24), where the float spacing is 1: its low bits are the
 // rounded integer, exact for |c q| < 2^22) and added with the native shared-memory integer add
 // (the FP32 add is a compare-and-swap loop with a round trip per attempt); zero contributions are
@@ -122,8 +122,8 @@ __device__ __forceinline__ void jdep(double* a, double c, double w)
 }
 template <int D>
 struct JScale {
-    static constexpr int nmin = D == 3 ? 256 : 512;
-    static constexpr float range = D == 3 ? 536870912.0f : 2147483648.0f - 2097152.0f;   // 2^29; 2^31 (1 - 2^-10)
+    static constexpr int nmin = D == 2 ? 512 : 256;
+    static constexpr float range = D == 2 ? 2147483648.0f - 2097152.0f : 536870912.0f;   // 2^31 (1 - 2^-10); 2^29
 };
 
 // Global chunk k of a launch group -> simulation, tile and particle slots.  Chunks are
@@ -169,7 +169,7 @@ __device__ __forceinline__ int warp_reserve(int tile, int* cursors)
 // ---- momentum updates; h = q dt / 2 (q = -1, m = 1, c = 1) ----------------------------
 
 // Boris: electric half kick, rotation about B by 2 atan(|h B|/gamma^-), electric half kick.
-template <int D, typename R>
+template <typename R>
 __device__ __forceinline__ void boris_update(R u[3], const R E[3], const R B[3], R h)
 {
     R um[3];
@@ -178,8 +178,7 @@ __device__ __forceinline__ void boris_update(R u[3], const R E[3], const R B[3],
     const R tf = h * m_rsqrt(R(1) + um[0] * um[0] + um[1] * um[1] + um[2] * um[2]);   // h / gamma^-
     const R tv[3] = {tf * B[0], tf * B[1], tf * B[2]};
     const R t2 = tv[0] * tv[0] + tv[1] * tv[1] + tv[2] * tv[2];
-    // (the FP32 3D push keeps the division, as it keeps phi_closed_log)
-    const R sf = D == 3 && sizeof(R) == 4 ? R(2) / (R(1) + t2) : R(2) * m_inv(R(1) + t2);
+    const R sf = R(2) / (R(1) + t2);
     const R up[3] = {um[0] + (um[1] * tv[2] - um[2] * tv[1]), um[1] + (um[2] * tv[0] - um[0] * tv[2]),
                      um[2] + (um[0] * tv[1] - um[1] * tv[0])};
     const R sv[3] = {sf * tv[0], sf * tv[1], sf * tv[2]};
@@ -448,7 +447,7 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
                 // ---- momentum update, charge -1, mass 1 (u^{n-1/2} -> u^{n+1/2}) ----
                 if (S.pusher == 1) vay_update<R>(u, E, B, hq);
                 else if (S.pusher == 2) higuera_cary_update<R>(u, E, B, hq);
-                else boris_update<D, R>(u, E, B, hq);
+                else boris_update<R>(u, E, B, hq);
                 const R ig = m_rsqrt(R(1) + u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);   // 1 / gamma
                 const R v[3] = {u[0] * ig, u[1] * ig, u[2] * ig};
 
