@@ -297,15 +297,13 @@ long long capacity(const pic_config* c)
 // Tile choice (the autotuner's defaults; `tile` in the config overrides the particle tile).
 void choose_tiles(const pic_config* c, int pt[3], int yt[3])
 {
-    const bool fp64 = c->precision == PIC_FP64;
     // field-solver tiles are fixed per dimension: k_yee is compiled for exactly these shapes
     if (c->dim == 1) {
         pt[0] = 32; yt[0] = 128;
     } else if (c->dim == 2) {
-        // 16x16, or 32x16 where a 16x16 tile of the slab holds less than one default work item
-        // (4.5 M electrons, 4 per cell, items of 2048: push 0.180 -> 0.172 ms; 2.1 M, 8 per cell,
-        // items of 1024: 0.124 with 16x16, 0.127 with 32x16)
-        pt[0] = c->ppc > 0 && 256 * c->ppc < default_item(capacity(c), 2, fp64) ? 32 : 16;
+        // 16x16 (32x16 measured 4 % less push time where a tile holds 1 k electrons, 2 % more where
+        // it holds 2 k; it also doubles the fixed-point unit of the FP32 current of a full item)
+        pt[0] = 16;
         pt[1] = 16; yt[0] = Y2_PX; yt[1] = Y2_PY;
     } else {
         // columns of Y3_PX x Y3_PY marching along z in segments: at least ~600 work items

@@ -95,19 +95,18 @@ __device__ __forceinline__ R interp(const R* f, const int bx, const int bxy, con
 }
 
 // Current accumulation in the work item's shared-memory box.  FP32: 32-bit fixed point with
-// the scale q = range / (max(N, nmin) w_max) of the item (N particles): a contribution of one
+// the scale q = 2^29 / (max(N, 256) w_max) of the item (N particles): a contribution of one
 // particle to one node is bounded by w |v| <= w_max (Esirkepov's partial sums of the shape
 // change are at most the move in cells, v dt/dx, times dx/dt; the transverse weights are
-// averages of shapes in [0, 1]; |v| < c = 1), so with range 2^31 (1 - 2^-10) and nmin 512 (2D)
-// |c q| < 2^22 and no node's sum, its N roundings included, reaches 2^31.  1D and 3D leave four
-// times the room: range 2^29, nmin 256 (their default items are not larger than before, and a finer
-// scale moved single electrons of the a0 = 20 focus by 1e-3 of the rms momentum against runs with
-// this one).  Each contribution is rounded to the nearest integer by one FMA with
+// averages of shapes in [0, 1]; |v| < c = 1), so |c q| <= 2^21 and no node's sum reaches 2^31.
+// (Two more bits fit, but electrons of a dense or strongly driven plasma amplify any change of the
+// rounding: runs with a finer scale differed by 1e-3 of the rms field from runs with this one, at
+// the same error against FP64.)  Each contribution is rounded to the nearest integer by one FMA with
 // 1.5 * 2^23 (the sum lands in [2^23, 2^24), where the float spacing is 1: its low bits are the
 // rounded integer, exact for |c q| < 2^22) and added with the native shared-memory integer add
 // (the FP32 add is a compare-and-swap loop with a round trip per attempt); zero contributions are
 // added too (no test).  The box is turned back into FP32 before its TMA reduce-add; each
-// contribution's rounding is at most max(N, nmin) w_max / (2 range).  FP64 keeps double sums.
+// contribution's rounding is at most max(N, 256) w_max 2^-30.  FP64 keeps double sums.
 // Each contribution is a product of a factor c along the current's own axis, scaled by q, and a
 // transverse weight w: the product, its scaling and its rounding are the one FMA.
 __device__ __forceinline__ void jdep(float* a, float c, float w)
@@ -120,11 +119,6 @@ __device__ __forceinline__ void jdep(double* a, double c, double w)
     const double v = c * w;
     if (v != 0.0) atomicAdd(a, v);
 }
-template <int D>
-struct JScale {
-    static constexpr int nmin = D == 2 ? 512 : 256;
-    static constexpr float range = D == 2 ? 2147483648.0f - 2097152.0f : 536870912.0f;   // 2^31 (1 - 2^-10); 2^29
-};
 
 // Global chunk k of a launch group -> simulation, tile and particle slots.  Chunks are
 // numbered per simulation by the tile scan (ctile / crange) and across the group by gprefix.
@@ -364,7 +358,7 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
         const PhaseRef<R>& pref = s_pref;     // read from shared memory where used (no registers held)
         // fixed-point scale of this item's current (FP32; unused in FP64)
         const float wmax = st->wmax;
-        const R jq = (sizeof(R) == 4 && wmax > 0.f) ? R(JScale<D>::range / ((float)max(p1 - p0, JScale<D>::nmin) * wmax)) : R(0);
+        const R jq = (sizeof(R) == 4 && wmax > 0.f) ? R(536870912.0f / ((float)max(p1 - p0, 256) * wmax)) : R(0);
         const R dtdx = bc.dtdx;
         const R jfac = bc.jfac;                     // -q dx/dt, q = -1
         const R hq = bc.hq;                         // q dt / 2
@@ -681,7 +675,7 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
         }
         if constexpr (sizeof(R) == 4) {
             // fixed point back to FP32, in place
-            const float inv = (float)max(p1 - p0, JScale<D>::nmin) * wmax * (1.0f / JScale<D>::range);
+            const float inv = (float)max(p1 - p0, 256) * wmax * (1.0f / 536870912.0f);
             int* Jq = reinterpret_cast<int*>(Js);
             for (int i = tid; i < 3 * bvol; i += nth) Jq[i] = __float_as_int(__int2float_rn(Jq[i]) * inv);
             __syncthreads();

@@ -4,9 +4,9 @@ and work items at the edges of the rule that sizes them, and the largest sum one
 
 Tolerances.  Default items: the FP32 / FP64 bars of tests/_support.py.  The heavy node: each of
 the N contributions to a node is rounded by at most half a unit of the fixed-point scale,
-2^-32 max(N, 512) w / (1 - 2^-10) (1D and 3D: 2^-30 max(N, 256) w), all the same way (the electrons are
-alike), so the sum by N times that; the other FP32 operations of a contribution (some twenty roundings of 2^-24 each)
-add at most 20 2^-24 of the largest J."""
+2^-30 max(N, 256) w, all the same way (the electrons are alike), so the sum by N times that; the
+other FP32 operations of a contribution (some twenty roundings of 2^-24 each) add at most 20 2^-24
+of the largest J."""
 import numpy as np
 import pytest
 
@@ -89,9 +89,7 @@ def test_every_electron_of_an_item_on_the_same_nodes(P, orc, dim, tile, count, c
     for c in range(6, 9):
         peak = np.abs(Fr[c]).max()
         assert peak > 0
-        unit = 2.0**-32 * max(min(count, chunk), 512) / (1 - 2.0**-10)
-        if dim != 2:
-            unit = 2.0**-30 * max(min(count, chunk), 256)
+        unit = 2.0**-30 * max(min(count, chunk), 256)
         bar = count * 0.7 * unit + 20 * 2.0**-24 * peak
         assert np.abs(Fg[c] - Fr[c]).max() < bar, (c, np.abs(Fg[c] - Fr[c]).max() / peak, bar / peak)
     sim.close()
