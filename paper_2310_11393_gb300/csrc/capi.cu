@@ -52,9 +52,10 @@ static void host_parallel(long long n, long long per_min, F body)
 
 int default_item(long long n, int dim, bool fp64)
 {
-    const long long slots = 152LL * (fp64 ? (dim == 1 ? 2 : 1) : (dim == 3 ? 2 : 4));
+    const int round = fp64 ? PUSH_ROUND_FP64 : 256;
+    const long long slots = 152LL * (fp64 ? (dim == 1 ? 4 : (dim == 2 ? 3 : 2)) : (dim == 3 ? 2 : 4));
     const long long per = (n + 4 * slots - 1) / (4 * slots);
-    return (int)std::min<long long>(ITEM_MAX, std::max<long long>(256, (per + 255) / 256 * 256));
+    return (int)std::min<long long>(ITEM_MAX, std::max<long long>(round, (per + round - 1) / round * round));
 }
 
 long long new_group_id()

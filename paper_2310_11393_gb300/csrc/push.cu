@@ -232,16 +232,20 @@ __device__ __forceinline__ void higuera_cary_update(R u[3], const R E[3], const 
 
 // Threads of a push block and blocks per SM the registers are budgeted for.  The 3D FP32
 // push shares its 101 KB box (16x8x4 tiles) among 512 threads at 64 registers: two blocks
-// keep 32 warps per SM busy instead of 16 with 256-thread blocks at 128 registers.
+// keep 32 warps per SM busy instead of 16 with 256-thread blocks at 128 registers.  The FP64 push is
+// bound by the FP64 pipe (two lanes per SM and clock), which four warps fill: blocks of 128 threads
+// leave small runs twice the items to spread over the SMs (1D, 57 k electrons: step 0.0285 -> 0.0265
+// ms; 2D, 131 k: 0.338 -> 0.333; 64 threads: 0.0262 and 0.329, but the 125 places of the 3D
+// histogram want a thread each).
 template <int D, typename R>
 __host__ __device__ constexpr int push_threads()
 {
-    return (D == 3 && sizeof(R) == 4) ? 512 : 256;
+    return sizeof(R) == 8 ? PUSH_ROUND_FP64 : (D == 3 ? 512 : 256);
 }
 template <int D, typename R>
 __host__ __device__ constexpr int push_min_blocks()
 {
-    return sizeof(R) == 8 ? 1 : (D <= 2 ? 4 : 2);
+    return sizeof(R) == 8 ? (D == 3 ? 2 : (D == 2 ? 3 : 4)) : (D <= 2 ? 4 : 2);
 }
 
 // Chunk k of a single simulation (its chunks are numbered from gprefix[0]).
@@ -364,16 +368,16 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
         const R hq = bc.hq;                         // q dt / 2
         const int hx[3] = {4, 2, 2};                // box halo below the tile per axis
 
-        // Rounds of nth particles (256 or 512).  Thread t takes particle t of the round: the
+        // Rounds of nth particles (128, 256 or 512).  Thread t takes particle t of the round: the
         // placement below writes a warp's particles into consecutive slots in lane order, so
         // slots that started as 32 consecutive cells (k_place_slab) stay close to that, whatever
         // the plasma does, and the loads are coalesced.  With a cell sort the P particles of a
         // cell (1, 2, 4 or 8) sit next to each other instead: lane l of warp w then takes particle
         // P l + (w mod P) of the round's (w div P)-th group of 32 P.  Either way a stencil node of
         // the deposit and the gather is mostly a different shared-memory word in every lane.
-        const int P = S.lane_p, wq = tid >> 5;
+        const int P = sizeof(R) == 8 ? min(S.lane_p, nth >> 5) : S.lane_p, wq = tid >> 5;
         int q = (tid & 31) * P + (wq & (P - 1)) + 32 * P * (wq / P);
-        if (S.pt[0] == 16 && P > 1 && P <= 4) {
+        if (sizeof(R) == 4 && S.pt[0] == 16 && P > 1 && P <= 4) {
             // 16-cell tile rows: a warp's 32 cells span two rows.  The box row pitch is 24
             // words, so rows two apart start 16 banks apart: the warp's groups take rows
             // (r, r + 2) of the round instead of (r, r + 1), and its two half-warps hit

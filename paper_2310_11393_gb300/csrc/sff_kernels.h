@@ -19,6 +19,7 @@ constexpr int COMP_TOTAL = 18, NFCOMP_INC = 24;
 __host__ __device__ constexpr int comp_eb(int parity) { return 6 * parity; }
 __host__ __device__ constexpr int comp_j(int parity) { return 12 + 3 * parity; }
 
+constexpr int PUSH_ROUND_FP64 = 128;    // threads of an FP64 push block
 constexpr int NCOUNTERS = 5;
 
 // One launch group: simulations of one dimension and precision advanced together.

@@ -71,9 +71,9 @@ struct pic_sim {
 
 // Particles per push work item when the configuration leaves it open, for n particles: about four
 // items for every block that the GPU holds at once (152 SMs; blocks per SM by registers and shared
-// memory), a multiple of 256 (a block's round), at most ITEM_MAX.  With fewer items than that the
-// last ones of a launch leave most SMs idle, below that the per-item set-up (the box load, the
-// clearing and the flush of the current) shows.  Push at the focus, items of 256 / 512 / 1024 /
+// memory), a multiple of a block's round (256; FP64 128), at most ITEM_MAX.  With fewer items than
+// that the last ones of a launch leave most SMs idle, below that the per-item set-up (the box load,
+// the clearing and the flush of the current) shows.  Push at the focus, items of 256 / 512 / 1024 /
 // 2048: 2D 14 k electrons 0.018 / 0.025 / 0.028 / 0.034 ms, 2D FP64 131 k 0.34 / 0.36 / 0.40 /
 // 0.65 ms, 3D 89 k 0.039 / 0.040 / 0.048 / - ms, 2D 2.1 M - / 0.127 / 0.124 / 0.146 ms, 3D 2.0 M
 // - / 0.368 / 0.337 / 0.327 ms, 2D 4.5 M - / 0.204 / 0.181 / 0.180 ms.
