@@ -915,7 +915,7 @@ pic_status pic_init(const pic_config* cfg_in, const pic_allocator* alloc, void* 
     const int bs = std::max(1, scatter_blocks_per_sm(cfg->dim, cfg->precision));
     g.inc_any = h.incgrid;
     g.scan_blocks = h.nscanblk;
-    g.tail = step_has_tail(L.nptiles);
+    g.tail = step_has_tail(L.nptiles, L.pt[0] * L.pt[1] * L.pt[2]);
     g.cellscan_grid = std::max(1, std::min(L.nptiles, 8 * nsm));
     g.inc_segs = (cfg->n[0] + 1 + 255) / 256;
     g.inc_rows = (cfg->dim > 1 ? cfg->n[1] + 1 : 1) * (cfg->dim > 2 ? cfg->n[2] + 1 : 1);

@@ -124,9 +124,14 @@ int device_sms();
 
 // Do the tile scan (one block per simulation) and the step end ride on the field solver's launch?
 // They save two launches and a fork of the step graph, some 4 us of a step; one block scans 4096
-// tiles in about 10 us beside a field solve of at least that size.  Larger simulations scan over
-// several blocks in a launch of their own.
-inline bool step_has_tail(int nptiles) { return nptiles <= 4096; }
+// tiles in about 10 us beside the field solve.  Up to 16384 tiles it still ends first where they
+// are of 256 cells or more (8192 of 16x16: scan 20 us, solve 45 us; the step of a 2D run of 2.1 M
+// cells and 4.5 M electrons 0.231 -> 0.2255 ms); beyond, and with smaller tiles, the scan goes over
+// several blocks in a launch of its own.
+inline bool step_has_tail(int nptiles, int tile_cells)
+{
+    return nptiles <= 4096 || (nptiles <= 16384 && tile_cells >= 256);
+}
 
 // Is field-solver tile t a work item?  In 2D and 3D a tile (column) whose first point lies on
 // the node line / plane x = n_x (or y = n_y), which holds nothing else, is not: the one before

@@ -1,5 +1,5 @@
 """The routes of a step and of the state's input and output: many steps in one graph launch, the tile
-scan on the field solver's launch up to 4096 tiles and beside it above, particles and fields through
+scan on the field solver's launch and in one of its own, particles and fields through
 more pieces than fit the staging memory at once.
 
 Tolerances.  Steps: the FP32 / FP64 bars of tests/_support.py against the oracle.  Input and output: a
@@ -49,11 +49,12 @@ def test_many_steps_in_one_call(P, orc, calls, sort_every):
     sim.close()
 
 
-@pytest.mark.parametrize("n", [(256, 256, 1), (257, 256, 1)])     # 4096 and 4160 tiles of 4x4 cells
+@pytest.mark.parametrize("n,tile", [((256, 256, 1), (4, 4)), ((257, 256, 1), (4, 4)),        # 4096, 4160 tiles
+                                    ((1040, 1025, 1), (16, 16)), ((1040, 1025, 1), (8, 8))])  # 4225, 16770 tiles
 @pytest.mark.parametrize("precision", [synth.FP32, synth.FP64])
-def test_tile_scan_with_and_beside_the_field_solver(P, orc, n, precision):
-    w = small_2d(precision=precision, steps=20).with_(n=n, slab_hi=(n[0] - 4, n[1] - 4, 1), ppc=1)
-    sim = P.Simulation(P.config_from(w, tile=(4, 4)))
+def test_tile_scan_with_and_beside_the_field_solver(P, orc, n, tile, precision):
+    w = small_2d(precision=precision, steps=20).with_(n=n, slab_hi=(n[0] - 4, 100, 1), ppc=1)
+    sim = P.Simulation(P.config_from(w, tile=tile))
     ref = orc.Sim(orc.config_from(w))
     sim.step(w.steps)
     ref.step(w.steps)
