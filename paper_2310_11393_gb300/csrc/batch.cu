@@ -113,14 +113,13 @@ pic_status build_entry(const std::vector<pic_sim*>& sims, BatchEntry** out, std:
         // own would take smaller items; the chunk tables hold these larger ones)
         long long total = 0;
         for (int i : mem) total += sims[i]->pcap;
-        const int item = default_item(total, kv.first.first, kv.first.second == PIC_FP64);
         std::vector<SimDev> hs(n);
         std::vector<Work> yw;
         yw.reserve(nyw);
         for (int k = 0; k < n; ++k) {
             pic_sim* s = sims[mem[k]];
             hs[k] = s->h;
-            if (s->cfg.chunk == 0) hs[k].chunk = std::max(s->h.chunk, item);
+            hs[k].chunk = std::max(s->h.chunk, work_item(&s->cfg, total));
             for (int t = 0; t < s->h.nytiles; ++t)
                 if (yee_tile_active(s->h, s->cfg.dim, t)) yw.push_back({k, t});
         }

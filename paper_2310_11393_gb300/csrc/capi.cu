@@ -58,6 +58,12 @@ int default_item(long long n, int dim, bool fp64)
     return (int)std::min<long long>(ITEM_MAX, std::max<long long>(round, (per + round - 1) / round * round));
 }
 
+int work_item(const pic_config* c, long long n)
+{
+    const int d = default_item(n, c->dim, c->precision == PIC_FP64);
+    return c->chunk == 0 ? d : (c->precision == PIC_FP64 ? std::min<int>(c->chunk, d) : c->chunk);
+}
+
 long long new_group_id()
 {
     static std::atomic<long long> next{1};
@@ -369,7 +375,7 @@ Layout make_layout(const pic_config* c)
     L.cap = capacity(c);
     L.max_exits = c->max_exits > 0 ? c->max_exits : L.cap;
     L.chunk = c->chunk > 0 ? c->chunk : ITEM_MAX;
-    L.item = c->chunk > 0 ? c->chunk : default_item(L.cap, c->dim, c->precision == PIC_FP64);
+    L.item = work_item(c, L.cap);
     L.max_chunks = (int)(L.nptiles + (L.cap + L.item - 1) / L.item + 1);
     // Every tile keeps slack for the particles within one cell outside it, the only ones a
     // step can bring in (a move is under one cell per axis).  With tiles at least two cells

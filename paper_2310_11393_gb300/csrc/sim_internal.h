@@ -79,6 +79,10 @@ struct pic_sim {
 // - / 0.368 / 0.337 / 0.327 ms, 2D 4.5 M - / 0.204 / 0.181 / 0.180 ms.
 constexpr int ITEM_MAX = 2048;
 int default_item(long long n, int dim, bool fp64);
+// ... and with the configuration's limit.  An FP64 item never gets larger than the default: one that
+// spans a dense tile leaves its block's four warps the last at work (1D plane wave at step 1800,
+// 32 768 electrons in tiles of 16 cells, limit 2048: step 0.0472 -> 0.0276 ms).
+int work_item(const pic_config* c, long long n);
 
 // a fresh launch-group id (never 0; never reused in the process)
 long long new_group_id();
