@@ -117,7 +117,7 @@ __device__ __forceinline__ void jdep(float* a, float c, float w)
 __device__ __forceinline__ void jdep(double* a, double c, double w)
 {
     const double v = c * w;
-    if (v != 0.0) atomicAdd(a, v);
+    if (nonzero(v)) atomicAdd(a, v);
 }
 
 // Global chunk k of a launch group -> simulation, tile and particle slots.  Chunks are
@@ -233,9 +233,9 @@ __device__ __forceinline__ void higuera_cary_update(R u[3], const R E[3], const 
 // Threads of a push block and blocks per SM the registers are budgeted for.  The 3D FP32
 // push shares its 101 KB box (16x8x4 tiles) among 512 threads at 64 registers: two blocks
 // keep 32 warps per SM busy instead of 16 with 256-thread blocks at 128 registers.  The FP64 push is
-// bound by the FP64 pipe (two lanes per SM and clock), which four warps fill: blocks of 128 threads
-// leave small runs twice the items to spread over the SMs (1D, 57 k electrons: step 0.0285 -> 0.0265
-// ms; 2D, 131 k: 0.338 -> 0.333; 64 threads: 0.0262 and 0.329, but the 125 places of the 3D
+// bound by the FP64 pipe (two lanes per SM and clock); blocks of 128 threads leave small runs twice
+// the items to spread over the SMs (1D, 32 768 electrons: step 0.0285 -> 0.0265 ms; 2D, 131 k: 0.338
+// -> 0.333; 64 threads: 0.0262 and 0.329, but the 125 places of the 3D
 // histogram want a thread each).
 template <int D, typename R>
 __host__ __device__ constexpr int push_threads()
@@ -281,7 +281,8 @@ __device__ __forceinline__ ChunkRef chunk_of_one(const SimDev& S, const int* __r
 // Fewer instructions beside it (the transverse weight as A A' + DS DS'/12, one FMA per
 // contribution, loads and adds at immediate offsets, one count per particle from which the tile
 // and frame counts follow): 3D push of 16.8 M electrons (tiles 16x8x4) 2.01 -> 1.84 ms, of 2.0 M
-// (tiles 8x8x8) 0.534 -> 0.450 ms, 2D of 2.1 M (tiles 32x16) 0.137 -> 0.133 ms.
+// (tiles 8x8x8) 0.534 -> 0.450 ms, 2D of 2.1 M (tiles 32x16) 0.137 -> 0.133 ms.  Consecutive slots
+// per warp, the quotients of the closed form and 16x8x4 default tiles since: 1.74, 0.325 and 0.121.
 template <int D, typename R, bool ONE, int BX, int BY>
 __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const SimDev& one, int nsims,
                                           const int* __restrict__ gprefix, int* __restrict__ counter, int sorting)
@@ -414,8 +415,8 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
 #pragma unroll
                 for (int d = 0; d < 3; ++d) {
                     if (d < D) {
-                        const int h = o[d] >= R(0.5);
-                        shape2(o[d] - R(h), Wp[d]);
+                        const int h = ge_half(o[d]);
+                        shape2(o[d] - flag(R(0), h), Wp[d]);
                         lp[d] = c[d] + h - 1 - T0[d] + hx[d];
                         shape2(o[d] - R(0.5), Wd[d]);
                         ld[d] = c[d] - 1 - T0[d] + hx[d];
@@ -465,11 +466,12 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
 #pragma unroll
                 for (int d = 0; d < D; ++d) {
                     mv[d] = dtdx * v[d];
-                    const int h0 = o[d] >= R(0.5);
-                    const R d0 = o[d] - R(h0);
+                    const int h0 = ge_half(o[d]);
+                    const R d0 = o[d] - flag(R(0), h0);
                     const R r1 = d0 + mv[d];
-                    const int sh = (int)m_floor(r1 + R(0.5));
-                    const R d1 = r1 - R(sh);
+                    R fsh;
+                    const int sh = floor_unit(r1 + R(0.5), fsh);
+                    const R d1 = r1 - (sizeof(R) == 4 ? R(sh) : fsh);
                     R w0[3], w1[3];
                     shape2(d0, w0);
                     shape2(d1, w1);
@@ -495,10 +497,10 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
 #pragma unroll
                 for (int d = 0; d < D; ++d) {
                     const R x = o[d] + mv[d];
-                    const R fl = m_floor(x);
+                    R fl;
+                    int k = floor_unit(x, fl);
                     R r = x - fl;
-                    int k = (int)fl;
-                    if (r >= R(1)) {
+                    if (ge_one(r)) {
                         r -= R(1);
                         k += 1;
                     }
@@ -694,7 +696,7 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
             const long long jbase = (long long)comp_j(par) * S.sc;
             for (int i = tid; i < 3 * bvol; i += nth) {
                 const R val = Js[i];
-                if (val != R(0)) {
+                if (nonzero(val)) {
                     const int comp = i / bvol, rem = i - comp * bvol;
                     const int lz = rem / bxy, rxy = rem - lz * bxy, ly = rxy / bx, lx = rxy - ly * bx;
                     atomicAdd(&Fg[jbase + comp * S.sc + (long long)(org[2] + lz) * S.sz +
