@@ -79,11 +79,11 @@ SLAB_CELLS = 0
 # ncu capture summarised in profiles/ (kept in step with the kernel: set to None when the
 # kernel changes and until it is captured again)
 PROFILED_TRAFFIC = {
-    ("2d_lp_1024sq", "k_push1<2,float>"): (108.4e6, "profiles/k_push_2d_lp_1024sq.md, step 762 (focus)"),
+    ("2d_lp_1024sq", "k_push1<2,float>"): (109.4e6, "profiles/k_push_2d_lp_1024sq.md, step 762 (focus)"),
     # the full 3D state (14 GB) is too large for a multi-pass capture: the box halved per axis
     # (2.1 M electrons, step 233 at the focus), scaled by the electrons (x8): the push's traffic
     # is per particle (record read and written) plus the grid per cell, both x8
-    ("3d_rp_512x256x256", "k_push1<3,float>"): (8 * 161.3e6, "profiles/k_push_3d_rp_256x128x128.md, box halved per "
+    ("3d_rp_512x256x256", "k_push1<3,float>"): (8 * 158.7e6, "profiles/k_push_3d_rp_256x128x128.md, box halved per "
                                                              "axis at the focus, scaled x8 by electrons and cells"),
 }
 
@@ -368,12 +368,22 @@ def run_ours(args, rank, world, local_rank):
                       "cell_updates_per_s": cells * args.steps * world / t_max,
                       "l2": "inputs larger than L2 (device state %.2f GB > 129 MB)" % (info.params.device_bytes / 1e9),
                       "parallelism": f"replicas x{world}" if world > 1 else "single GPU", "tiles": tune},
-           # kernels launched by the timed run: per step push, tile scan, field solve, step end
-           # (+ the incident field on the grid; + cell count, cell scan and scatter on cell-sort
-           # steps), and one k_prefix before the first step
-           "roofline": roof, "clocks": clk, "gpu_launches": (5 if w.incident_grid else 4) * args.steps + 1
-           + (3 * (args.steps // prm.sort_every) if prm.sort_every > 0 else 0), "e2e": e2e}
+           "roofline": roof, "clocks": clk, "gpu_launches": launches(w, prm, args.steps), "e2e": e2e}
     return out
+
+
+def launches(w, prm, steps):
+    """Kernels launched by the timed run: per step push and field solve, which takes the tile scan
+    and the step end along up to 4096 tiles (16384 of 256 cells); two more where it does not (+ the
+    incident field on the grid; + cell count, cell scan and scatter on cell-sort steps), and one
+    k_prefix before the first step."""
+    tiles, cells = 1, 1
+    for d in range(w.dim):
+        tiles *= -(-w.n[d] // prm.tile[d])
+        cells *= prm.tile[d]
+    tail = tiles <= 4096 or (tiles <= 16384 and cells >= 256)
+    sorts = steps // prm.sort_every if prm.sort_every > 0 else 0
+    return (2 if tail else 4) * (steps - sorts) + 7 * sorts + (steps if w.incident_grid else 0) + 1
 
 
 def run_e2e(args, w, cfg, pic, torch, stream, alloc, snap, s0):

@@ -117,8 +117,8 @@ typedef struct {
     uint64_t seed;           /* SplitMix64 seed of the slab positions */
     int64_t max_particles;   /* particle capacity; 0: slab count (pic_set_particles may need more) */
     int64_t max_exits;       /* exit-record capacity; 0: max_particles */
-    int32_t chunk;           /* particles per push work item (multiple of 256, 256..16384); 0: 2048, or
-                                fewer where that leaves the GPU too few work items */
+    int32_t chunk;           /* particles per push work item (multiple of 256, 256..16384; FP64: at
+                                most); 0: 2048, or fewer where that leaves the GPU too few work items */
     int32_t pusher;          /* PIC_PUSHER_*: momentum update of the Lorentz force (Sec. 2 cites all three) */
     int32_t profile;         /* PIC_PROFILE_*; the super-Gaussian uses prof_order (p >= 1), prof_x0,
                                 prof_fwhm (> 0) and prof_cut, all in code units along x */

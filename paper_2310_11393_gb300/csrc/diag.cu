@@ -124,7 +124,7 @@ __device__ __forceinline__ bool incident_zero(int beam, int comp)
 // A block takes 256 points of a row at a time: one double-precision phase reference per row
 // segment (per point and component it was most of the kernel: FP64 runs at 1/64 of the FP32
 // rate), the components in turn, those that are identically zero without the closed form.
-// Double sums.  3D RP 512 x 256 x 256: 12.0 -> 6.6 ms with the particle part.
+// Double sums.  3D RP 512 x 256 x 256: 12.0 -> 4.8 ms with the particle part.
 template <int D, typename R>
 __global__ void __launch_bounds__(256) k_energy_fields(const SimDev* __restrict__ sim, double* __restrict__ acc)
 {
@@ -230,7 +230,7 @@ __device__ __forceinline__ void hist_add(double* bins, double ux, double uy, dou
 
 // The same for single-precision momenta: the bin from FP32 arithmetic wherever that cannot differ
 // from the double one, i.e. unless it comes within its error of a bin's edge (2.1 M electrons,
-// 96 x 36 bins: 0.53 -> 0.2 ms; the double functions run at 1/64 of the FP32 rate).  Errors:
+// 96 x 36 bins: 0.53 -> 0.10 ms; the double functions run at 1/64 of the FP32 rate).  Errors:
 // gamma - 1 = u^2/(gamma + 1) within 8 roundings of 2^-24 relative; the angle within 8 of pi.
 __device__ __forceinline__ void hist_add(double* bins, float ux, float uy, float uz, float w, int n_e, double e_max,
                                          int n_a)
@@ -310,7 +310,8 @@ __global__ void k_eval_incident(const SimDev* __restrict__ sim, long long n, con
 // piece of staging memory at a time, and the copy engine moves host doubles: 64 B per electron
 // and 72 B per grid point at the link's rate (190-200 GB/s to and from host pages that are mapped
 // already) instead of a pass of host threads over freshly mapped buffers.  Read-back of 2.1 M
-// electrons 15-22 -> 1.5 ms, of 12 small simulations 21 -> 3 ms.
+// electrons 15-22 -> 4 ms, of 12 small simulations with their fields 21 -> 9 ms (what is left is
+// mapping the caller's fresh output pages).
 
 // first[t]: particles of the tiles before t in buffer set par, first[nptiles] their total
 __global__ void __launch_bounds__(1024) k_tile_first(const SimDev* __restrict__ sim, int par, int* __restrict__ first)

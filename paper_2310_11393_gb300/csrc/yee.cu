@@ -599,7 +599,7 @@ __global__ void __launch_bounds__(NT, 2) k_yee2r1(const __grid_constant__ SimDev
 // iteration q runs A(q+1) together with D(q-1), then B(q+1): two barriers per plane.  A thread
 // keeps its own point's E, Bh and N of the planes on the way in registers; shared memory serves
 // the neighbours' values (21 loads per point and plane, 39 without), and the loop is unrolled over
-// the ring: 0.617 -> 0.589 ms on 512 x 256 x 256.  What bounds it now is the chain of two barriers
+// the ring: 0.617 -> 0.555 ms on 512 x 256 x 256.  What bounds it now is the chain of two barriers
 // per plane at 24 warps per SM (issue slots 67 % busy while a block runs, DRAM 2.6 of 6.8 TB/s):
 // leaving out the loads and the clearing of J where no electron is (80 % of this box) changed
 // nothing (0.594 against 0.600 ms).

@@ -1,5 +1,6 @@
 """The branch-free FP32 reciprocal, square root, quotient and inverse square root of the incident
-field against IEEE arithmetic, over every mantissa.
+field against IEEE arithmetic, over every mantissa, and the FP64 push's decisions by bits (zero, half,
+one, floor of a move) against the comparisons they stand for: exact.
 
 Tolerances.  One Newton step from an estimate of relative error e < 2^-22 leaves an error of at most
 2^-44, so a result differs from the correctly rounded one only where the value lies within 2^-44 of
@@ -24,6 +25,25 @@ __global__ void k(int op, int n, const float* x, const float* y, float* r)
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     r[i] = op == 0 ? sff::m_inv(x[i]) : op == 1 ? sff::m_root(x[i]) : op == 2 ? sff::m_quot(y[i], x[i]) : sff::m_isqrt(x[i]);
+}
+__global__ void kb(int n, const double* x, int* r, double* f)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int k = sff::floor_unit(x[i], f[i]);
+    r[i] = (k + 1) | (sff::nonzero(x[i]) << 4) | (sff::ge_half(x[i]) << 5) | (sff::ge_one(x[i]) << 6);
+}
+extern "C" int bits(int n, const double* x, int* r, double* f)
+{
+    char* d;
+    if (cudaMalloc(&d, 20ll * n)) return 1;
+    cudaMemcpy(d, x, 8ll * n, cudaMemcpyHostToDevice);
+    kb<<<(n + 255) / 256, 256>>>(n, (const double*)d, (int*)(d + 16ll * n), (double*)(d + 8ll * n));
+    cudaMemcpy(f, d + 8ll * n, 8ll * n, cudaMemcpyDeviceToHost);
+    cudaMemcpy(r, d + 16ll * n, 4ll * n, cudaMemcpyDeviceToHost);
+    const int e = (int)cudaGetLastError();
+    cudaFree(d);
+    return e;
 }
 extern "C" int run(int op, int n, const float* x, const float* y, float* r)
 {
@@ -67,3 +87,19 @@ def test_every_mantissa(lib, op, exponent):
     off = np.abs(r.view(np.int32).astype(np.int64) - want.view(np.int32))
     assert off.max() <= 1
     assert np.count_nonzero(off) <= n * 2.0**-16
+
+
+def test_decisions_by_bits(lib):
+    edges = np.array([-1.0, -0.5, 0.0, 0.5, 1.0, 2.0])
+    x = np.concatenate([edges, np.nextafter(edges, 9), np.nextafter(edges, -9), [-0.0, 1e-310, -1e-310],
+                        np.random.default_rng(6).uniform(-1, 2, 100001)])
+    x = np.concatenate([x[(x >= -1) & (x < 2)], [np.nan, -np.nan]])
+    r, fl = np.empty(len(x), np.int32), np.empty(len(x))
+    p = ctypes.c_void_p
+    assert lib.bits(len(x), x.ctypes.data_as(p), r.ctypes.data_as(p), fl.ctypes.data_as(p)) == 0
+    k = np.nan_to_num(np.floor(x)).astype(int)
+    np.testing.assert_array_equal((r & 15) - 1, k)
+    np.testing.assert_array_equal(fl, k)
+    np.testing.assert_array_equal((r >> 4) & 1, x != 0)
+    np.testing.assert_array_equal((r >> 5) & 1, x >= 0.5)
+    np.testing.assert_array_equal((r >> 6) & 1, x >= 1)

@@ -36,9 +36,9 @@ def _compare(sim, ref, w, steps, prec):
 
 
 @pytest.mark.parametrize("calls", [(64,), (79,), (3, 64, 1, 12), (63,)])
-@pytest.mark.parametrize("sort_every", [0, 5])
-def test_many_steps_in_one_call(P, orc, calls, sort_every):
-    w = small_2d(precision=synth.FP64)
+@pytest.mark.parametrize("sort_every,ppc", [(0, 4), (5, 4), (5, 8)])     # (lane strides 1, 4, 4 of 128 threads)
+def test_many_steps_in_one_call(P, orc, calls, sort_every, ppc):
+    w = small_2d(precision=synth.FP64).with_(ppc=ppc)
     sim = P.Simulation(P.config_from(w, sort_every=sort_every))
     ref = orc.Sim(orc.config_from(w))
     for n in calls:
