@@ -1003,7 +1003,13 @@ __device__ __forceinline__ void yee3s_body(const SimDev* __restrict__ sims, cons
             return;
         }
         if (nwork <= nblk) break;
-        if (tid == 0) s_item = nblk + atomicAdd(counter, 1);
+        if (tid == 0) {
+            s_item = nblk + atomicAdd(counter, 1);
+            // The output slots start over with every item (slot 1 first), and a segment of an odd
+            // number of planes ends on slot 1: its last store has to have read that before the
+            // next item's first plane is written (no cost: three planes lie between them)
+            bulk_wait_read0();
+        }
         __syncthreads();
         item = s_item;
         __syncthreads();
