@@ -107,8 +107,9 @@ __device__ __forceinline__ R interp(const R* f, const int bx, const int bxy, con
 // (the FP32 add is a compare-and-swap loop with a round trip per attempt); zero contributions are
 // added too (no test).  The box is turned back into FP32 before its TMA reduce-add; each
 // contribution's rounding is at most max(N, 256) w_max 2^-30.  FP64 keeps double sums.
-// Each contribution is a product of a factor c along the current's own axis, scaled by q, and a
-// transverse weight w: the product, its scaling and its rounding are the one FMA.
+// A contribution is a product c w; its scaling by q and its rounding are one FMA: 1D and 2D fold q into
+// the factor c along the current's own axis, w the transverse weight; 3D (FP32) takes the rounded sum
+// of Esirkepov's terms for c and q for w (see `line` below).
 __device__ __forceinline__ void jdep(float* a, float c, float w)
 {
     const float f = fmaf(c, w, 12582912.0f);
@@ -455,10 +456,19 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
                 // core nodes m = 0, 1, 2); the new shape is shifted by sh in {-1, 0, 1} nodes
                 // (|move| < 1 cell), so a lane that changes its nearest node has one node more, two
                 // past the middle one on the side it moves to (m = 3).  A / DS: mean of old and new
-                // shape / shape change on these nodes.  Along the current's own axis the running sum
-                // of DS ends at zero, so that component has the core nodes 0 and 1, and a lane that
-                // crosses a third, with the charge -/+ DS[3] that it carries over it.  The additions
-                // at nodes that only crossing lanes have are left to those lanes.
+                // shape (TERMS: old shape) / shape change on these nodes.  Along the current's own axis
+                // the running sum of DS ends at zero, so that component has the core nodes 0 and 1, and
+                // a lane that crosses a third, with the charge -/+ DS[3] that it carries over it.  The
+                // additions at nodes that only crossing lanes have are left to those lanes.
+                //
+                // TERMS, the 3D FP32 push: the transverse weight as the four terms of Esirkepov's sum and
+                // the current as the running sum of products with it, each operation rounded where and
+                // in the order it was in the builds up to 70273bb.  The shorter forms below equal these
+                // but for the last bit, which puts one node in a hundred of a tile on the neighbouring
+                // integer; the electrons of the 3D run at a0 = 20 (16.8 M, 150 steps) amplified that to
+                // momenta 1.2e-6 rms and up to 1.3e-3 off, twice and more what two runs of one build
+                // differ by.  3D push of 16.8 M electrons 1.74 -> 1.82 ms, of 2.0 M 0.325 -> 0.334 ms.
+                constexpr bool TERMS = D == 3 && sizeof(R) == 4;
                 R A[3][4], DS[3][4];
                 int jb = 0;                                  // core node (0, 0, 0) in the box
                 bool cross[3] = {false, false, false}, low[3] = {false, false, false};
@@ -483,10 +493,10 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
 #pragma unroll
                     for (int m = 0; m < 3; ++m) {
                         DS[d][m] = n1[m] - w0[m];
-                        A[d][m] = w0[m] + R(0.5) * DS[d][m];
+                        A[d][m] = TERMS ? w0[m] : w0[m] + R(0.5) * DS[d][m];
                     }
                     DS[d][3] = n1[3];
-                    A[d][3] = R(0.5) * n1[3];
+                    A[d][3] = TERMS ? R(0) : R(0.5) * n1[3];
                     jb += (c[d] + h0 - 1 - T0[d] + hx[d]) * (d == 0 ? 1 : (d == 1 ? bx : bxy));
                 }
                 // ---- move: carry the offset into the cell index; removal near the faces.
@@ -548,9 +558,9 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
                 }
                 // ---- the deposit on the nodes set up above ----
                 // Esirkepov's transverse weight S0 S0' + (DS S0' + S0 DS')/2 + DS DS'/3 is
-                // A A' + DS DS'/12; along the current's own axis the factor is the running sum
-                // of DS, times the scale of the fixed point (FP32)
-                const R qs = sizeof(R) == 4 ? jq : R(1);
+                // A A' + DS DS'/12 (without TERMS); along the current's own axis the factor is the
+                // running sum of DS, times the scale of the fixed point (FP32)
+                const R qs = sizeof(R) == 4 && !TERMS ? jq : R(1);
                 const R cw = jfac * wt * qs;
                 const R t12 = R(1) / R(12);
                 const int pitch[3] = {1, bx, bxy};
@@ -560,18 +570,45 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
                 // node m of axis d as an offset from core node 0
                 auto at = [&](int d, int m) { return m < 3 ? m * pitch[d] : ex[d]; };
                 // the current along axis d at the nodes of transverse weight w from f on
-                auto line = [&](int d, R* f, const R C[3], R w) {
-                    jdep(f, C[0], w);
-                    jdep(f + pitch[d], C[1], w);
-                    if (cross[d]) jdep(f + (low[d] ? -pitch[d] : 2 * pitch[d]), C[2], w);
+                auto line = [&](int d, R* f, const R C[4], R w) {
+                    if constexpr (TERMS) {
+                        const float e = __fmul_rn(C[3], w), v0 = fmaf(C[0], w, e), v1 = fmaf(C[1], w, v0);
+                        jdep(f, v0, jq);
+                        jdep(f + pitch[d], v1, jq);
+                        if (cross[d])
+                            jdep(f + (low[d] ? -pitch[d] : 2 * pitch[d]), low[d] ? e : fmaf(C[2], w, v1), jq);
+                    } else {
+                        jdep(f, C[0], w);
+                        jdep(f + pitch[d], C[1], w);
+                        if (cross[d]) jdep(f + (low[d] ? -pitch[d] : 2 * pitch[d]), C[2], w);
+                    }
                 };
-                auto run_sum = [&](int d, R C[3]) {
-                    C[0] = cw * (DS[d][0] + (low[d] ? DS[d][3] : R(0)));
-                    C[1] = C[0] + cw * DS[d][1];
-                    C[2] = cw * (low[d] ? DS[d][3] : -DS[d][3]);
+                // TERMS: the charge moved to nodes 0, 1, 2 and (crossing downwards) the one before node 0
+                auto run_sum = [&](int d, R C[4]) {
+                    if constexpr (TERMS) {
+#pragma unroll
+                        for (int m = 0; m < 3; ++m) C[m] = cw * DS[d][m];
+                        C[3] = low[d] ? cw * DS[d][3] : R(0);
+                    } else {
+                        C[0] = cw * (DS[d][0] + (low[d] ? DS[d][3] : R(0)));
+                        C[1] = C[0] + cw * DS[d][1];
+                        C[2] = cw * (low[d] ? DS[d][3] : -DS[d][3]);
+                    }
+                };
+                // transverse weight of node m of axis t and node k of axis z (dk = DS'/12)
+                auto trans = [&](int t, int m, int z, int k, R dk) -> R {
+                    if constexpr (TERMS) {
+                        const float third = 1.0f / 3.0f;
+                        float w = __fmul_rn(0.5f * DS[t][m], A[z][k]);
+                        w = fmaf(A[t][m], A[z][k], w);
+                        w = fmaf(0.5f * A[t][m], DS[z][k], w);
+                        return fmaf(third * DS[t][m], DS[z][k], w);
+                    } else {
+                        return A[t][m] * A[z][k] + DS[t][m] * dk;
+                    }
                 };
                 if constexpr (D == 1) {
-                    R C[3];
+                    R C[4];
                     run_sum(0, C);
                     R* f = Js + jb;
                     line(0, f, C, R(1));
@@ -586,7 +623,7 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
 #pragma unroll
                     for (int d = 0; d < 2; ++d) {
                         const int t = 1 - d;
-                        R C[3];
+                        R C[4];
                         run_sum(d, C);
                         R* f = Js + d * bvol + jb;
 #pragma unroll
@@ -608,7 +645,7 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
 #pragma unroll
                     for (int d = 0; d < 3; ++d) {
                         const int t = d == 0 ? 1 : 0, z = d == 2 ? 1 : 2;       // transverse axes
-                        R C[3];
+                        R C[4];
                         run_sum(d, C);
                         R* f = Js + d * bvol + jb;
 #pragma unroll
@@ -618,7 +655,7 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
 #pragma unroll
                             for (int b = 0; b < 4; ++b)
                                 if (b < 3 || cross[t])
-                                    line(d, f + at(z, k) + at(t, b), C, A[t][b] * A[z][k] + DS[t][b] * dk);
+                                    line(d, f + at(z, k) + at(t, b), C, trans(t, b, z, k, dk));
                         }
                     }
                 }
