@@ -314,7 +314,8 @@ void choose_tiles(const pic_config* c, int pt[3], int yt[3])
         pt[1] = 16; yt[0] = Y2_PX; yt[1] = Y2_PY;
     } else {
         // columns of Y3_PX x Y3_PY marching along z in segments: at least ~600 work items
-        // (a few per resident block on a full GPU), segments of at most 64 planes
+        // (a few per resident block on a full GPU), segments of at most 64 planes (more only by
+        // the rule below)
         // particle tiles: rows of 16 cells in a box of 24 words a row spread the shared-memory
         // banks; rows of 8 in a box of 16 use half of them (push of 2.0 M electrons at the focus:
         // 8x8x8 0.469 ms, 8x8x4 0.451, 16x8x4 0.327, 16x4x4 0.328, 32x4x2 0.337)
@@ -325,6 +326,8 @@ void choose_tiles(const pic_config* c, int pt[3], int yt[3])
         int nseg = std::max<int>(ceil_div(nz, 64), (int)std::min<long long>(nz, (600 + ncol - 1) / ncol));
         nseg = std::min(nseg, std::max(1, nz / 8));
         yt[2] = ceil_div(nz, nseg);
+        // never plane n_z as a segment of its own: its Mur condition needs E of plane n_z - 1
+        while (yt[2] < nz && c->n[2] % yt[2] == 0) ++yt[2];
     }
     for (int d = c->dim; d < 3; ++d) pt[d] = yt[d] = 1;
     for (int d = 0; d < c->dim; ++d)

@@ -35,3 +35,10 @@ def test_segments_of_odd_length_one_after_another(P, orc, prec):
     params = P.pic_derive_params(P.config_from(small_3d().with_(n=n, ppc=0)))
     assert params.yee_tile[2] == 13
     _check(P, orc, n, prec, 4)
+
+
+@pytest.mark.parametrize("prec", [synth.FP32, synth.FP64])
+@pytest.mark.parametrize("n", [(72, 72, 72), (64, 24, 81), (40, 48, 126)])
+def test_last_plane_of_the_box(P, orc, n, prec):
+    """Grids whose segments would leave the plane z = n_z to one of its own."""
+    _check(P, orc, n, prec, 5)
