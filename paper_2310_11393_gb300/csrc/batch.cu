@@ -184,6 +184,7 @@ pic_status build_entry(const std::vector<pic_sim*>& sims, BatchEntry** out, std:
     }
     // the plain step, and (when a member sorts by cell) the cell-sort step
     for (int v = 0; v < (e->sort_every > 0 ? 2 : 1); ++v) {
+        cudaGetLastError();      // (an error of an earlier call of the caller's is not one of these launches)
         if (cudaStreamBeginCapture(e->cs, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
             err = "batch capture could not start";
             free_entry(e);
@@ -212,7 +213,8 @@ pic_status build_entry(const std::vector<pic_sim*>& sims, BatchEntry** out, std:
         }
         cudaGraph_t* gp = v == 1 ? &e->sort_graph : &e->graph;
         cudaGraphExec_t* xp = v == 1 ? &e->sort_exec : &e->exec;
-        const cudaError_t ec = cudaStreamEndCapture(e->cs, gp);
+        const cudaError_t el = cudaGetLastError(), ec = cudaStreamEndCapture(e->cs, gp);
+        if (ce == cudaSuccess) ce = el;
         if (ce == cudaSuccess) ce = ec;
         if (ce == cudaSuccess) ce = cudaGraphInstantiate(xp, *gp, 0);
         if (ce != cudaSuccess) {

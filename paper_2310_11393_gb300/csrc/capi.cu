@@ -532,6 +532,7 @@ constexpr int MANY_STEPS = 16;
 pic_status capture_step(pic_sim* s, bool sorted, int steps, GraphBundle* out)
 {
     cudaStream_t cs = s->cap_stream, cs2 = s->cap_stream2;
+    cudaGetLastError();      // (an error of an earlier call of the caller's is not one of these launches)
     CU_CHECK(s, cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
     if (s->grp.tail && !sorted) {
@@ -554,17 +555,20 @@ pic_status capture_step(pic_sim* s, bool sorted, int steps, GraphBundle* out)
         if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, s->ev_join, 0);
         launch_step_end(s->grp, cs);
     }
+    const cudaError_t el = cudaGetLastError();      // of the launches: a graph without one of them is no step
+    if (e == cudaSuccess) e = el;
     cudaGraph_t g = nullptr;
     const cudaError_t ec = cudaStreamEndCapture(cs, &g);
     if (e == cudaSuccess) e = ec;
-    if (e != cudaSuccess && g) {
-        cudaGraphDestroy(g);
-        g = nullptr;
+    cudaGraphExec_t x = nullptr;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&x, g, 0);
+    if (e != cudaSuccess) {
+        if (g) cudaGraphDestroy(g);
+        cudaGetLastError();
+        return fail(s, PIC_ECUDA, "graph capture failed: %s", cudaGetErrorString(e));
     }
-    if (e != cudaSuccess) return fail(s, PIC_ECUDA, "graph capture failed: %s", cudaGetErrorString(e));
     out->graph = g;
-    e = cudaGraphInstantiate(&out->exec, g, 0);
-    if (e != cudaSuccess) return fail(s, PIC_ECUDA, "graph instantiate failed: %s", cudaGetErrorString(e));
+    out->exec = x;
     return PIC_OK;
 }
 
@@ -950,12 +954,17 @@ pic_status pic_step(pic_sim* s, int n_steps, void* stream)
     if (n_steps > 0) ensure_prefix(s, st);
     int i = 0;
     if (s->grp.tail && s->sort_every <= 0 && n_steps >= 4 * MANY_STEPS) {
-        // (not while the caller captures the stream: only its launches belong there)
+        // captured at the first such call (not while the caller captures the stream: only its launches
+        // belong there; not with another device current than the simulation's).  Where that fails the
+        // steps go one by one
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        int dev = -1;
         CU_CHECK(s, cudaStreamIsCapturing(st, &cap));
-        if (!s->many_graph.exec && cap == cudaStreamCaptureStatusNone) {
-            const pic_status r = capture_step(s, false, MANY_STEPS, &s->many_graph);
-            if (r != PIC_OK) return r;
+        if (!s->many_graph.exec && !s->many_failed && cap == cudaStreamCaptureStatusNone &&
+            cudaGetDevice(&dev) == cudaSuccess && dev == s->device) {
+            const std::string before = s->err;
+            s->many_failed = capture_step(s, false, MANY_STEPS, &s->many_graph) != PIC_OK;
+            if (s->many_failed) s->err = before;
         }
         if (s->many_graph.exec)
             for (; i + MANY_STEPS <= n_steps; i += MANY_STEPS) CU_CHECK(s, cudaGraphLaunch(s->many_graph.exec, st));

@@ -17,6 +17,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <mutex>
 
 #include "beam.cuh"
 #include "sched.cuh"
@@ -1496,6 +1497,17 @@ void launch_sort_linear(const SimDev* sim, int dim, int prec, long long n, cudaS
     SFF_DISPATCH(dim, prec, sortlin_t, sim, n, s);
 }
 
+// Every simulation and batch of a dimension, precision and box pitch launches the same kernel, some of
+// them long after they were set up: the kernel's limit of dynamic shared memory is only ever raised.
+template <typename K>
+static void raise_smem(K k, size_t smem)
+{
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lk(mu);
+    cudaFuncAttributes a;
+    if (cudaFuncGetAttributes(&a, k) == cudaSuccess && (size_t)a.maxDynamicSharedSizeBytes < smem)
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
 template <int D, typename R>
 struct PushAttr {
     size_t smem;
@@ -1505,8 +1517,8 @@ struct PushAttr {
     {
         auto k = k_push<D, R, BX, BY>;
         auto k1 = k_push1<D, R, BX, BY>;
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        raise_smem(k, smem);
+        raise_smem(k1, smem);
         int a = 0, b = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k, push_threads<D, R>(), smem);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k1, push_threads<D, R>(), smem);

@@ -51,6 +51,7 @@ struct pic_sim {
     unsigned long long* d_bits = nullptr;
     GraphBundle step_graph;
     GraphBundle many_graph;      // MANY_STEPS steps (captured when a call first asks for a few times that)
+    bool many_failed = false;    // ... could not be
     // id of the launch group whose chunk numbering and work counters are set for this sim's
     // current particle layout (each step ends by setting them for its own group; any other
     // change of the layout clears it, and the next step of a group starts with k_prefix)
