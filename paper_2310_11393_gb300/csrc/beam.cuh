@@ -200,7 +200,9 @@ __device__ __forceinline__ void poisson3_log(const BeamC<R>& b, Cx<R> tau, R lnw
 template <typename R>
 __device__ __forceinline__ bool phi_closed(const BeamC<R>& b, R rho2, R zeta, Cx<R> u, R uu, R tmz, R tpz, Cx<R> P[4])
 {
-    // R = sqrt(u) from |u| (no scaling needed: |u| lies between the ring's edge and the box)
+    // R = sqrt(u) from |u| (no scaling needed: |u| lies between the ring's edge and the box; where an
+    // FP32 |u|^2 overflows all the same, 4e9 a from the focus, the field is below 3e-10 of its peak)
+    if (sizeof(R) == 4 && uu > R(3e38)) return false;
     const R im = m_isqrt(uu), au = uu * im;       // 1/|u|, |u| = |R|^2
     const R hp = R(0.5) * (au + m_abs(u.x)), ih = m_isqrt(hp);
     const R big = hp * ih, small = R(0.5) * m_abs(u.y) * ih;
@@ -213,8 +215,8 @@ __device__ __forceinline__ bool phi_closed(const BeamC<R>& b, R rho2, R zeta, Cx
     const Cx<R> taum = {tmz - qq.x, -qq.y};
     const Cx<R> taup = {tpz + qq.x, b.two_a + qq.y};
     const R xm = w2m1(b, taum), xp = w2m1(b, taup);
-    const bool use_m = R(1) + xm < b.wcut;
-    const bool use_p = R(1) + xp < b.wcut && R(1) + xp < b.wrel * (R(1) + xm);
+    const bool use_m = !(R(1) + xm >= b.wcut);      // (a NaN goes into the field)
+    const bool use_p = !(R(1) + xp >= b.wcut) && !(R(1) + xp >= b.wrel * (R(1) + xm));
     if (!use_m && !use_p) return false;
     // G^(n)_pm = g^(n)(tau_+) +- g^(n)(tau_-)
     Cx<R> G0m = {0, 0}, G1p = {0, 0}, G1m = {0, 0}, G2p = {0, 0}, G2m = {0, 0};
@@ -264,8 +266,8 @@ __device__ __forceinline__ bool phi_closed_log(const BeamC<R>& b, R rho2, R zeta
     const Cx<R> taum = {tmz - qq.x, -qq.y};
     const Cx<R> taup = {tpz + qq.x, b.two_a + qq.y};
     const R xm = w2m1(b, taum), xp = w2m1(b, taup);
-    const bool use_m = R(1) + xm < b.wcut;
-    const bool use_p = R(1) + xp < b.wcut;
+    const bool use_m = !(R(1) + xm >= b.wcut);      // (a NaN goes into the field)
+    const bool use_p = !(R(1) + xp >= b.wcut);
     if (!use_m && !use_p) return false;
     Cx<R> g0m = {0, 0}, g1m = {0, 0}, g2m = {0, 0}, g0p = {0, 0}, g1p = {0, 0}, g2p = {0, 0};
     if (use_m) poisson3_log(b, taum, R(0.5) * m_log1p(xm), g0m, g1m, g2m);
