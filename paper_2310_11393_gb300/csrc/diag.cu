@@ -231,14 +231,16 @@ __device__ __forceinline__ void hist_add(double* bins, double ux, double uy, dou
 // The same for single-precision momenta: the bin from FP32 arithmetic wherever that cannot differ
 // from the double one, i.e. unless it comes within its error of a bin's edge (2.1 M electrons,
 // 96 x 36 bins: 0.53 -> 0.10 ms; the double functions run at 1/64 of the FP32 rate).  Errors:
-// gamma - 1 = u^2/(gamma + 1) within 8 roundings of 2^-24 relative; the angle within 8 of pi.
+// gamma - 1 = u^2/(gamma + 1) within 8 roundings of 2^-24 relative; the angle within 8 of pi.  The
+// double gamma - 1 has its own, of 2^-53 gamma: they count where the bins are that narrow.
 __device__ __forceinline__ void hist_add(double* bins, float ux, float uy, float uz, float w, int n_e, double e_max,
                                          int n_a)
 {
     const float up2 = uy * uy + uz * uz, u2 = ux * ux + up2;
-    const float fe = u2 / (1.0f + sqrtf(1.0f + u2)) * ((float)n_e / (float)e_max);
+    const float scale = (float)n_e / (float)e_max;
+    const float fe = u2 / (1.0f + sqrtf(1.0f + u2)) * scale;
     const float fa = atan2f(sqrtf(up2), ux) * ((float)n_a * 0.318309886f);
-    const float de = 1e-6f * fe + 1e-30f, da = 2e-6f * (float)n_a;
+    const float de = 1e-6f * fe + 4.5e-16f * scale, da = 2e-6f * (float)n_a;
     const float ie = floorf(fe), ia = floorf(fa);
     const bool sure = fe - ie > de && fe - ie < 1.0f - de && fa - ia > da && fa - ia < 1.0f - da && u2 < 1e30f;
     if (!sure || n_e > (1 << 16) || n_a > (1 << 16)) {
