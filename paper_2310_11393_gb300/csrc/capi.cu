@@ -318,8 +318,11 @@ void choose_tiles(const pic_config* c, int pt[3], int yt[3])
         // the rule below)
         // particle tiles: rows of 16 cells in a box of 24 words a row spread the shared-memory
         // banks; rows of 8 in a box of 16 use half of them (push of 2.0 M electrons at the focus:
-        // 8x8x8 0.469 ms, 8x8x4 0.451, 16x8x4 0.327, 16x4x4 0.328, 32x4x2 0.337)
-        pt[0] = 16; pt[1] = 8; pt[2] = 4;
+        // 8x8x8 0.469 ms, 8x8x4 0.451, 16x8x4 0.327, 16x4x4 0.328, 32x4x2 0.337).  Where the
+        // configuration sets the tile along some axes only, the others get 8 cells (a box of 16 cells
+        // along x may not fit the shared memory beside them)
+        const bool open = c->tile[0] == 0 && c->tile[1] == 0 && c->tile[2] == 0;
+        pt[0] = open ? 16 : 8; pt[1] = 8; pt[2] = open ? 4 : 8;
         yt[0] = Y3_PX; yt[1] = Y3_PY;
         const long long ncol = (long long)ceil_div(c->n[0] + 1, Y3_PX) * ceil_div(c->n[1] + 1, Y3_PY);
         const int nz = c->n[2] + 1;
