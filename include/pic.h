@@ -361,8 +361,8 @@ pic_status pic_serve_close(pic_server* srv);
  * the status word and take a zero prefix, which keeps every later offset inside the
  * particle arrays (the particle layout is then wrong, and the next synchronous call returns
  * PIC_ETIMEOUT).  block = -1 restores publishing.  Only simulations with more than 4096
- * particle tiles use the multi-block scan.  Synchronous.  Errors: PIC_EINVAL (spins < 1),
- * PIC_ECUDA. */
+ * particle tiles have the multi-block scan (up to 16384 tiles of 256 cells or more they use it
+ * from this call on).  Synchronous.  Errors: PIC_EINVAL (spins < 1), PIC_ECUDA. */
 pic_status pic_test_hold_scan(pic_sim* sim, int block, int spins);
 
 /* ---- measurement aid (no counterpart in the paper) -------------------------------- */

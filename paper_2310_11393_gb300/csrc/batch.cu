@@ -163,7 +163,7 @@ pic_status build_entry(const std::vector<pic_sim*>& sims, BatchEntry** out, std:
             g.inc_rows = std::max(g.inc_rows, (c.dim > 1 ? c.n[1] + 1 : 1) * (c.dim > 2 ? c.n[2] + 1 : 1));
         }
         g.tail = true;
-        for (int i : mem) g.tail &= sff::step_has_tail(sims[i]->h.nptiles, sims[i]->h.pt[0] * sims[i]->h.pt[1] * sims[i]->h.pt[2]);
+        for (int i : mem) g.tail &= sims[i]->grp.tail;
         const int nsm = prop.multiProcessorCount;
         const int bp = std::max(1, sff::prepare_push(g.dim, g.prec, g.push_bx, g.push_by, psm));
         const int byy = std::max(1, sff::prepare_yee(g.dim, g.prec, ysm));

@@ -1071,6 +1071,18 @@ pic_status pic_test_hold_scan(pic_sim* s, int block, int spins)
     static_assert(offsetof(SimDev, scan_hold) == offsetof(SimDev, scan_spins) + sizeof(int), "layout");
     CU_CHECK(s, cudaMemcpy(reinterpret_cast<char*>(s->d) + o, reinterpret_cast<const char*>(&s->h) + o, 2 * sizeof(int),
                            cudaMemcpyHostToDevice));
+    // where one block of the field solver's launch scans the tiles instead, the steps go over to
+    // the scan that this call is about
+    if (s->h.nscanblk > 1 && s->grp.tail) {
+        CU_CHECK(s, cudaDeviceSynchronize());
+        for (GraphBundle* g : {&s->step_graph, &s->many_graph}) {
+            if (g->exec) cudaGraphExecDestroy(g->exec);
+            if (g->graph) cudaGraphDestroy(g->graph);
+            *g = GraphBundle{};
+        }
+        s->grp.tail = false;
+        return capture_step(s, false, 1, &s->step_graph);
+    }
     return PIC_OK;
 }
 
