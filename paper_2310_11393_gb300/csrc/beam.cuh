@@ -251,11 +251,11 @@ __device__ __forceinline__ bool phi_closed(const BeamC<R>& b, R rho2, R zeta, Cx
 
 // The same from hypot, atan2 and log1p of the library and correctly rounded reciprocals and
 // roots: the FP32 pushes.  Electrons of a strong focus amplify a last-bit change of the incident
-// field up to 1e4-fold within 100 steps, so the form above, though no less accurate and 2 to 3 %
-// of a step faster, moved single electrons by 1e-3 .. 1e-2 of the rms momentum in 8 of 41 sampled
-// runs; this one leaves as many outside as two runs of one build differ in (2).  With the
-// quotients and roots of m_inv, m_root and m_quot a 2D LP step takes 0.142 ms (1.05 M cells, 10
-// electrons per cell; with the compiler's 0.147).
+// field up to 1e4-fold within 100 steps: the form above, though no less accurate and 2 to 3 % of a
+// step faster, moved single electrons by 1e-3 .. 1e-2 of the rms momentum in 8 of 41 sampled runs.
+// This one gives bit for bit what the compiler's divisions and roots give (the momenta of 590 000
+// electrons after their first push, RP and LP); with m_inv, m_root and m_quot in their place a 2D LP
+// step takes 0.142 ms (1.05 M cells, 8 electrons per slab cell; with the compiler's 0.147).
 template <typename R>
 __device__ __forceinline__ bool phi_closed_log(const BeamC<R>& b, R rho2, R zeta, Cx<R> u, R tmz, R tpz, Cx<R> P[4])
 {

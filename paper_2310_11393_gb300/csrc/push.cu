@@ -237,8 +237,11 @@ __device__ __forceinline__ void higuera_cary_update(R u[3], const R E[3], const 
 // keep 32 warps per SM busy instead of 16 with 256-thread blocks at 128 registers.  The FP64 push is
 // bound by the FP64 pipe (two lanes per SM and clock); blocks of 128 threads leave small runs twice
 // the items to spread over the SMs (1D, 32 768 electrons: step 0.0285 -> 0.0265 ms; 2D, 131 k: 0.338
-// -> 0.333; 64 threads: 0.0262 and 0.329, but the 125 places of the 3D
-// histogram want a thread each).
+// -> 0.333; 64 threads: 0.0262 and 0.329, but the 125 places of the 3D histogram want a thread
+// each).  In 3D the registers allow two FP64 blocks on an SM, the box of 202 KB one; four warps on it
+// are still faster than the eight of earlier builds (tiles 8x8x8; RP runs around the focus: 0.6 M
+// electrons at 4 per cell 2.37 -> 2.02 ms a step, 0.08 M at 2 per cell 0.78 -> 0.44, 0.4 M at 1 per
+// cell 1.78 -> 1.67).
 template <int D, typename R>
 __host__ __device__ constexpr int push_threads()
 {
@@ -280,11 +283,11 @@ __device__ __forceinline__ ChunkRef chunk_of_one(const SimDev& S, const int* __r
 // wavefronts when the others leave it out: with the nodes of the deposit taken as three core nodes
 // per axis plus one for the lanes that cross (instead of a window of four for a warp with any
 // crossing lane) the adds' wavefronts fell from 36.2 M to 22.7 M in the 3D push of 2.1 M electrons.
-// Fewer instructions beside it (the transverse weight as A A' + DS DS'/12, one FMA per
-// contribution, loads and adds at immediate offsets, one count per particle from which the tile
-// and frame counts follow): 3D push of 16.8 M electrons (tiles 16x8x4) 2.01 -> 1.84 ms, of 2.0 M
-// (tiles 8x8x8) 0.534 -> 0.450 ms, 2D of 2.1 M (tiles 32x16) 0.137 -> 0.133 ms.  Consecutive slots
-// per warp, the quotients of the closed form and 16x8x4 default tiles since: 1.74, 0.325 and 0.121.
+// Beside it: loads and adds at immediate offsets, one count per particle from which the tile and
+// frame counts follow, consecutive slots per warp, quotients without range branches, in 1D and 2D the
+// transverse weight as A A' + DS DS'/12 and one FMA per contribution.  Push at the focus, before all
+// of this and with it: 3D of 16.8 M electrons (tiles 16x8x4) 2.00 -> 1.82 ms, 2D of 2.1 M (tiles
+// 32x16) 0.137 -> 0.120; 3D of 2.0 M from the former default tiles of 8x8x8 to 16x8x4 0.533 -> 0.338.
 template <int D, typename R, bool ONE, int BX, int BY>
 __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const SimDev& one, int nsims,
                                           const int* __restrict__ gprefix, int* __restrict__ counter, int sorting)
@@ -468,7 +471,7 @@ __device__ __forceinline__ void push_body(const SimDev* __restrict__ sims, const
                 // but for the last bit, which puts one node in a hundred of a tile on the neighbouring
                 // integer; the electrons of the 3D run at a0 = 20 (16.8 M, 150 steps) amplified that to
                 // momenta 1.2e-6 rms and up to 1.3e-3 off, twice and more what two runs of one build
-                // differ by.  3D push of 16.8 M electrons 1.74 -> 1.82 ms, of 2.0 M 0.325 -> 0.334 ms.
+                // differ by.  3D push of 16.8 M electrons 1.74 -> 1.82 ms, of 2.0 M 0.325 -> 0.338 ms.
                 constexpr bool TERMS = D == 3 && sizeof(R) == 4;
                 R A[3][4], DS[3][4];
                 int jb = 0;                                  // core node (0, 0, 0) in the box

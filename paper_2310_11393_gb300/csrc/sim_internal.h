@@ -71,8 +71,8 @@ struct pic_sim {
 
 
 // Particles per push work item when the configuration leaves it open, for n particles: about four
-// items for every block that the GPU holds at once (152 SMs; blocks per SM by registers and shared
-// memory), a multiple of a block's round (256; FP64 128), at most ITEM_MAX.  With fewer items than
+// items for every block that the GPU holds at once (152 SMs; blocks per SM by registers and, in FP32,
+// shared memory; 3D FP64 counts two, of which its box lets one run at a time), a multiple of a block's round (256; FP64 128), at most ITEM_MAX.  With fewer items than
 // that the last ones of a launch leave most SMs idle, below that the per-item set-up (the box load,
 // the clearing and the flush of the current) shows.  Push at the focus, items of 256 / 512 / 1024 /
 // 2048: 2D 14 k electrons 0.018 / 0.025 / 0.028 / 0.034 ms, 2D FP64 131 k 0.34 / 0.36 / 0.40 /

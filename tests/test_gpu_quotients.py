@@ -89,6 +89,19 @@ def test_every_mantissa(lib, op, exponent):
     assert np.count_nonzero(off) <= n * 2.0**-16
 
 
+@pytest.mark.parametrize("op", ["inv", "root", "quot"])
+def test_correctly_rounded(lib, op):
+    """Not one unit off: every mantissa of an even and an odd exponent (the reciprocal and the root repeat
+    beyond that), the quotient with a random numerator for each."""
+    n = 1 << 24
+    x = ((np.uint32(127) << np.uint32(23)) + np.arange(n, dtype=np.uint32)).view(np.float32)
+    y = np.random.default_rng(7).uniform(1.0, 4.0, n).astype(np.float32)
+    r = np.empty_like(x)
+    f = ctypes.POINTER(ctypes.c_float)
+    assert lib.run(["inv", "root", "quot"].index(op), n, x.ctypes.data_as(f), y.ctypes.data_as(f), r.ctypes.data_as(f)) == 0
+    np.testing.assert_array_equal(r, np.float32(1) / x if op == "inv" else np.sqrt(x) if op == "root" else y / x)
+
+
 def test_decisions_by_bits(lib):
     edges = np.array([-1.0, -0.5, 0.0, 0.5, 1.0, 2.0])
     x = np.concatenate([edges, np.nextafter(edges, 9), np.nextafter(edges, -9), [-0.0, 1e-310, -1e-310],
