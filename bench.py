@@ -83,7 +83,7 @@ PROFILED_TRAFFIC = {
     # the full 3D state (14 GB) is too large for a multi-pass capture: the box halved per axis
     # (2.1 M electrons, step 233 at the focus), scaled by the electrons (x8): the push's traffic
     # is per particle (record read and written) plus the grid per cell, both x8
-    ("3d_rp_512x256x256", "k_push1<3,float>"): (8 * 158.7e6, "profiles/k_push_3d_rp_256x128x128.md, box halved per "
+    ("3d_rp_512x256x256", "k_push1<3,float>"): (8 * 160.3e6, "profiles/k_push_3d_rp_256x128x128.md, box halved per "
                                                              "axis at the focus, scaled x8 by electrons and cells"),
 }
 

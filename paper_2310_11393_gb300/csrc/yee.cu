@@ -600,7 +600,7 @@ __global__ void __launch_bounds__(NT, 2) k_yee2r1(const __grid_constant__ SimDev
 // keeps its own point's E, Bh and N of the planes on the way in registers; shared memory serves
 // the neighbours' values (21 loads per point and plane, 39 without), and the loop is unrolled over
 // the ring: 0.617 -> 0.555 ms on 512 x 256 x 256.  What bounds it now is the chain of two barriers
-// per plane at 24 warps per SM (issue slots 67 % busy while a block runs, DRAM 2.6 of 6.8 TB/s):
+// per plane at 24 warps per SM (issue slots 53 % busy, DRAM 4.8 of the 6.8 TB/s of a copy):
 // leaving out the loads and the clearing of J where no electron is (80 % of this box) changed
 // nothing (0.594 against 0.600 ms).
 // Bh is kept for x in [x0-2, x0+PX], y in [y0-2, y0+PY] and planes from z0-1; N for x in
